@@ -586,11 +586,10 @@ int mdg_mlp_adam(mdg_mlp m, float lr, void* stream);
  * training uses mdg_mlp_set_train_path. */
 #define MDG_MLP_PATH_TCGEN05_PAIRS 2
 int mdg_mlp_set_path(mdg_mlp m, int32_t path);
-/* Training path of mdg_mlp_grad: MDG_MLP_PATH_TCGEN05 (default: every GEMM of the forward and
- * backward pass on tcgen05.mma with the accumulator in tensor memory, both operands K-major in
- * shared memory; the epilogues write the pre-activations, the SiLU activations and the
- * hidden gradients together with their transposes, which are the K-major operands of the
- * weight gradients dW = dZ^T X; those are split over the batch and added up with atomics) or
+/* Training path of mdg_mlp_grad: MDG_MLP_PATH_TCGEN05 (default: one kernel takes every 128-row
+ * tile through the forward and backward pass on tcgen05.mma with the accumulators in tensor
+ * memory, a second one forms the weight gradients dW = dZ^T H, split over the batch and added
+ * up with atomics; x and t 16-byte aligned) or
  * MDG_MLP_PATH_MMA_SYNC (the mma.sync GEMMs). Errors: MDG_ERR_ARG. */
 int mdg_mlp_set_train_path(mdg_mlp m, int32_t path);
 /* Bounds of the tcgen05 kernel's waits on its own mbarriers (its MMAs, bulk copies and

@@ -1,6 +1,6 @@
 // BF16 tensor-core kernels of the learned surrogate: a tiled GEMM on mma.sync
 // m16n8k16 (FP32 accumulation) with fused epilogues for the forward pass, the input
-// gradient and the weight gradient, the bias-gradient reduction, Adam, and the input
+// gradient and the weight gradient, the bias-gradient reduction, and the input
 // standardisation. The network is 64 -> 256 -> 256 -> 256 -> 32 (41 inputs and 13 outputs
 // used, zero padded), SiLU on the hidden layers.
 #include <cuda_bf16.h>
@@ -277,23 +277,6 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__
     }
 }
 
-// Adam (Kingma and Ba) on the flat FP32 master parameters; refreshes their bf16 copies.
-__global__ void adam_kernel(float* __restrict__ w, bf16* __restrict__ w16, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, long long n, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        w[i] = wi;
-        w16[i] = __float2bfloat16_rn(wi);
-    }
-}
-
 __global__ void to_bf16_kernel(const float* __restrict__ w, bf16* __restrict__ w16, long long n)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -364,15 +347,6 @@ cudaError_t mlp_backward(const MlpView& w, const void* x, int B, float* const z_
         }
     }
     return cudaSuccess;
-}
-
-cudaError_t mlp_adam(const MlpView& w, const float* grad, float* m, float* v, float lr, int step, cudaStream_t s)
-{
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    adam_kernel<<<152 * 4, 256, 0, s>>>(w.master, static_cast<bf16*>(w.w16), grad, m, v, MDG_MLP_PARAMS, lr, b1, b2,
-                                        eps, c1, c2);
-    return cudaGetLastError();
 }
 
 cudaError_t mlp_refresh_bf16(const MlpView& w, cudaStream_t s)

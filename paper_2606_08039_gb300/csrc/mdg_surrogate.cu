@@ -75,12 +75,7 @@ struct mdg_mlp_s {
     int wait_limit = MDG_MLP_DEFAULT_TRY_WAITS;  // bounded waits of the tcgen05 kernel
     int spin_limit = MDG_MLP_DEFAULT_POLLS;
     int train_path = MDG_MLP_PATH_TCGEN05;
-    __nv_bfloat16* hT[3] = {};  // tcgen05 training: transposed activations and gradients
-    __nv_bfloat16* dzT[3] = {};
-    __nv_bfloat16* dyT = nullptr;
-    __nv_bfloat16* xT = nullptr;
-    __nv_bfloat16* wT = nullptr;  // W2^T, W3^T, W4^T
-    bool wT_stale = true;
+    float* loss_part = nullptr;  // tcgen05 training: the loss's partial sums
     mdg::MlpView view() const { return layout(master, w16); }
 };
 
@@ -108,25 +103,25 @@ void destroy_mlp(mdg_mlp m)
     cudaFree(m->fb_count);
     cudaFree(m->status);
     cudaFree(m->img);
-    for (int l = 0; l < 3; ++l) {
-        cudaFree(m->hT[l]);
-        cudaFree(m->dzT[l]);
-    }
-    cudaFree(m->dyT);
-    cudaFree(m->xT);
-    cudaFree(m->wT);
+    cudaFree(m->loss_part);
     delete m;
 }
 
-// The tcgen05 kernel reads the weights from their image; rebuild it after they change.
+// The tcgen05 kernels read the weights from their image; rebuild it after mdg_mlp_set_params (Adam
+// refreshes it itself).
+cudaError_t refresh_image(mdg_mlp m, cudaStream_t s)
+{
+    if (!m->img_stale) return cudaSuccess;
+    const cudaError_t e = mdg::mlp_build_image(m->view(), m->img, s);
+    if (e == cudaSuccess) m->img_stale = false;
+    return e;
+}
+
 cudaError_t forward_umma(mdg_mlp m, const void* x, int B, float* y, uint32_t* status, cudaStream_t s,
                          const mdg::MlpApply* apply = nullptr)
 {
-    if (m->img_stale) {
-        cudaError_t e = mdg::mlp_build_image(m->view(), m->img, s);
-        if (e != cudaSuccess) return e;
-        m->img_stale = false;
-    }
+    const cudaError_t e = refresh_image(m, s);
+    if (e != cudaSuccess) return e;
     if (m->path == MDG_MLP_PATH_TCGEN05_PAIRS)
         return mdg::mlp_forward_umma_pairs(m->view(), m->img, x, B, y, status, m->wait_limit, m->spin_limit, s, apply);
     return mdg::mlp_forward_umma(m->view(), m->img, x, B, y, status, m->wait_limit, m->spin_limit, s);
@@ -176,7 +171,7 @@ int mdg_mlp_create(int32_t max_batch, const float* init, mdg_mlp* out)
         alloc((void**)&m->dz[l], B * H * 2);
     }
     alloc((void**)&m->y, B * MDG_MLP_OUT_PAD * 4);
-    alloc((void**)&m->dy, B * MDG_MLP_OUT_PAD * 2);
+    alloc((void**)&m->dy, B * 64 * 2);  // 64 columns on the tcgen05 training path
     alloc((void**)&m->x, B * MDG_MLP_IN_PAD * 2);
     alloc((void**)&m->loss, 4);
     alloc((void**)&m->norm, (4 * MDG_MLP_IN + 2 * MDG_MLP_OUT) * 4);
@@ -185,13 +180,7 @@ int mdg_mlp_create(int32_t max_batch, const float* init, mdg_mlp* out)
     alloc((void**)&m->fb_count, 4);
     alloc((void**)&m->status, 8);
     alloc((void**)&m->img, mdg::mlp_image_bytes());
-    for (int l = 0; l < 3; ++l) {
-        alloc((void**)&m->hT[l], B * H * 2);
-        alloc((void**)&m->dzT[l], B * H * 2);
-    }
-    alloc((void**)&m->dyT, B * MDG_MLP_OUT_PAD * 2);
-    alloc((void**)&m->xT, B * MDG_MLP_IN_PAD * 2);
-    alloc((void**)&m->wT, mdg::mlp_weights_transposed_elems() * 2);
+    alloc((void**)&m->loss_part, B / 16 * 4);
     if (e == cudaSuccess && init) e = cudaMemcpy(m->master, init, P * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = mdg::mlp_refresh_bf16(m->view(), 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -227,7 +216,6 @@ int mdg_mlp_set_params(mdg_mlp m, const float* host_in)
     cudaError_t e = cudaMemcpy(m->master, host_in, (size_t)MDG_MLP_PARAMS * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = mdg::mlp_refresh_bf16(m->view(), 0);
     m->img_stale = true;
-    m->wT_stale = true;
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_set_params");
 }
@@ -319,36 +307,32 @@ int mdg_mlp_grad(mdg_mlp m, const uint16_t* x, const float* t, int32_t B, float*
 {
     if (!m || !x || !t) return fail(MDG_ERR_ARG, "mdg_mlp_grad: NULL argument");
     if (!batch_ok(m, B)) return fail(MDG_ERR_ARG, "mdg_mlp_grad: B = %d must be a multiple of 128 <= %d", B, m->max_batch);
+    if (m->train_path == MDG_MLP_PATH_TCGEN05 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(t)) & 15u))
+        return fail(MDG_ERR_ARG, "mdg_mlp_grad: x and t must be 16-byte aligned");
     Guard g(m->device);
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(m->loss, 0, 4, s);
-    float* zs[3] = {m->z[0], m->z[1], m->z[2]};
-    void* hs[3] = {m->h[0], m->h[1], m->h[2]};
-    void* dzs[3] = {m->dz[0], m->dz[1], m->dz[2]};
+    cudaError_t e;
     if (m->train_path == MDG_MLP_PATH_TCGEN05) {
-        if (e == cudaSuccess && m->wT_stale) {
-            e = mdg::mlp_weights_transposed(m->view(), m->wT, s);
-            if (e == cudaSuccess) m->wT_stale = false;
-        }
         mdg::TrainBuffers tb;
         for (int l = 0; l < 3; ++l) {
             tb.z[l] = m->z[l];
             tb.h[l] = m->h[l];
-            tb.hT[l] = m->hT[l];
             tb.dz[l] = m->dz[l];
-            tb.dzT[l] = m->dzT[l];
         }
-        tb.y = m->y;
         tb.dy = m->dy;
-        tb.dyT = m->dyT;
-        tb.xT = m->xT;
-        tb.wT = m->wT;
-        if (e == cudaSuccess) e = mdg::mlp_grad_umma(m->view(), tb, x, B, t, m->loss, m->grad, m->status, s);
+        tb.loss = m->loss_part;
+        e = refresh_image(m, s);
+        if (e == cudaSuccess)
+            e = mdg::mlp_grad_umma(m->view(), m->img, tb, x, B, t, m->loss, loss_out, m->grad, m->status, s);
     } else {
+        float* zs[3] = {m->z[0], m->z[1], m->z[2]};
+        void* hs[3] = {m->h[0], m->h[1], m->h[2]};
+        void* dzs[3] = {m->dz[0], m->dz[1], m->dz[2]};
+        e = cudaMemsetAsync(m->loss, 0, 4, s);
         if (e == cudaSuccess) e = mdg::mlp_forward(m->view(), x, B, zs, hs, m->y, t, m->dy, m->loss, s);
         if (e == cudaSuccess) e = mdg::mlp_backward(m->view(), x, B, zs, hs, m->dy, dzs, m->grad, s);
+        if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToDevice, s);
     }
-    if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_grad");
 }
 
@@ -358,9 +342,8 @@ int mdg_mlp_adam(mdg_mlp m, float lr, void* stream)
     if (!(lr > 0.f)) return fail(MDG_ERR_ARG, "mdg_mlp_adam: lr must be > 0");
     Guard g(m->device);
     m->step += 1;
-    m->img_stale = true;
-    m->wT_stale = true;
-    cudaError_t e = mdg::mlp_adam(m->view(), m->grad, m->m, m->v, lr, m->step, (cudaStream_t)stream);
+    m->img_stale = false;  // Adam writes every weight's place in the image
+    cudaError_t e = mdg::mlp_adam(m->view(), m->img, m->grad, m->m, m->v, lr, m->step, (cudaStream_t)stream);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_adam");
 }
 

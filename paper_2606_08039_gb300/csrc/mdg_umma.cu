@@ -29,46 +29,22 @@
 // MDG_STATUS_TIMEOUT in the status word, every role leaves its loop, the copies and MMAs
 // already issued are waited for (again with a bound), the tensor memory is freed and the
 // block returns.
-#include <cuda.h>
-#include <cuda_bf16.h>
-#include <stdint.h>
-
-#include "mdg.h"
-#include "mdg_internal.cuh"
+#include "mdg_umma.cuh"
 
 namespace mdg {
 namespace {
 
-constexpr int kRows = 128;                 // tile rows (UMMA M)
-constexpr int kEpiWarps = 16;              // four per TMEM lane quadrant
 constexpr int kProdWarp = kEpiWarps;       // producer warp
 constexpr int kMmaWarp = kEpiWarps + 1;    // MMA warp (also allocates the tensor memory)
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kSlots = 4;
-constexpr uint32_t kSlotBytes = 32768;     // one [256 x 64] bf16 weight chunk
-constexpr uint32_t kChunkBytes = 16384;    // one [128 x 64] bf16 activation chunk
 constexpr uint32_t kOffAct = 0;            // activations [128 x 256]: four chunks
 constexpr uint32_t kOffX = 4 * kChunkBytes;  // inputs [128 x 64]: one chunk
 constexpr uint32_t kOffSlot = kOffX + kChunkBytes;
 constexpr uint32_t kDynBytes = kOffSlot + kSlots * kSlotBytes;
-constexpr uint32_t kTmemCols = 512;        // two accumulators of 256 columns
 constexpr int kLoadsPerTile = 10;          // W1, W2 chunks 0-3, W3 chunks 0-3, W4
-constexpr uint32_t kSuspendNs = 1000;      // longest suspension of one mbarrier try_wait
-constexpr int kWaitLimit = MDG_MLP_DEFAULT_TRY_WAITS;  // try_waits (at most ~0.26 s) before giving up
 
-// Weight image: the chunks in the order the MMAs consume them, load i at i * 32 KB.
-//   load 0      W1 [256 x 64]
-//   loads 1-4   W2 chunk c [256 x 64]
-//   loads 5-8   W3 chunk c [256 x 64]
-//   load 9      W4 [32 x 256] as four [32 x 64] chunks of 4 KB (16 KB)
-constexpr uint32_t kImgBytes = 9 * kSlotBytes + 16384;
-static_assert(kImgBytes == 2 * (256 * 64 + 2 * 256 * 256 + 32 * 256), "the image holds every weight once");
 static_assert(kDynBytes + 1024 + 4096 <= 232448, "shared memory of one block");
-
-__device__ __forceinline__ uint32_t image_layer_base(int l)
-{
-    return l == 0 ? 0u : l == 1 ? kSlotBytes : l == 2 ? 5 * kSlotBytes : 9 * kSlotBytes;
-}
 
 // mbarriers
 enum {
@@ -81,141 +57,6 @@ enum {
     kBarMmaDone = kBarActFull + 4,    // MMA commit at the end: nothing left in flight
     kNumBars
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr)
-{
-    uint64_t d = (uint64_t)((saddr & 0x3FFFF) >> 4);  // start address
-    d |= (uint64_t)1 << 16;                           // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1 << 46;                           // descriptor version
-    d |= (uint64_t)2 << 61;                           // 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor of kind::f16: bf16 A and B (K-major), FP32 D, M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16_ss(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accumulate)
-{
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-
-// The mbarrier completes once every tcgen05 operation issued so far by this thread is done.
-__device__ __forceinline__ void mma_commit(uint32_t mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(uint32_t mbar, uint32_t parity)
-{
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
-// Wait for the phase of `parity` to complete: one non-blocking test, then mbarrier.try_wait,
-// which suspends the thread in hardware until the phase completes or about kSuspendNs pass.
-// Gives up when another role has aborted (abort != null) or after `limit` tries, which
-// records the timeout and aborts the block. The work waits take the launch's limit; the
-// drain waits of the exit path always take kWaitLimit, so that a block leaves only once
-// every copy and MMA it issued has completed.
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int* abort, uint32_t* status,
-                                          int limit)
-{
-    if (mbar_test(mbar, parity)) return true;
-    for (int i = 0; i < limit; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity), "r"(kSuspendNs)
-            : "memory");
-        if (done) return true;
-        if (abort && *abort) return false;
-    }
-    if (abort) *abort = 1;
-    atomicOr(status, MDG_STATUS_TIMEOUT);
-    return false;
-}
-
-// The same for waits on the critical path between MMAs and epilogue: poll with test_wait
-// (a suspended thread wakes up later than a polling one), backing off by `sleep_ns` between
-// polls (0: none), at most `limit` polls.
-__device__ __forceinline__ bool mbar_spin(uint32_t mbar, uint32_t parity, volatile int* abort, uint32_t* status,
-                                          int sleep_ns, int limit)
-{
-    for (int i = 0; i < limit; ++i) {
-        if (mbar_test(mbar, parity)) return true;
-        if ((i & 63) == 63 && *abort) return false;
-        if (sleep_ns) __nanosleep(sleep_ns);
-    }
-    *abort = 1;
-    atomicOr(status, MDG_STATUS_TIMEOUT);
-    return false;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes) : "memory");
-}
-
-// Bulk copy global -> shared; completes `bytes` of the mbarrier's transaction count.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t s, const void* g)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(g));
-}
-
-// 16 (x16) or 8 (x8) consecutive FP32 accumulator columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8])
-{
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // SiLU of two pre-activations given as h = z/2: silu(z) = z / (1 + exp(-z)) = h (1 + tanh h),
 // one special-function instruction each (tanh.approx.f32, relative error about 2^-11).
@@ -506,29 +347,6 @@ enum {
 
 // Image index of load k of a pair: 0 W1; 1-4 W2 c0-3, 5 W2 c0; 6-9 W3 c0-3, 10 W3 c0; 11 W4.
 __device__ __forceinline__ int pair_load_image(int k) { return (int)((0x958765143210ull >> (4 * k)) & 15u); }
-
-// TMA of one [128 x 64] bf16 input tile (rows row..row+127) into 128-byte-swizzled shared
-// memory, completing on mbar; and its prefetch into L2.
-__device__ __forceinline__ void tma_rows(uint32_t dst, const CUtensorMap* map, int row, uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(mbar) : "memory");
-}
-__device__ __forceinline__ void tma_rows_prefetch(const CUtensorMap* map, int row)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];\n"
-                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t r[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
 
 template <bool kApply>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -844,277 +662,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
 }
 
-// ---- training GEMMs on tcgen05: C[M x N] = A[M x K] B[N x K]^T, both operands K-major ----
-//
-// One 128-thread block computes a 128 x BN tile of C over a range of K (split-K when
-// gridDim.z > 1: the partial tiles are added to the output with atomics). Per 64-wide K chunk
-// every thread copies its share of the A and B chunks into shared memory (cp.async, 16 bytes
-// each, written straight into the 128-byte-swizzled K-major layout of the inference kernel's
-// operands; a 32-wide last chunk is padded with zeros), one thread issues the chunk's four
-// tcgen05.mma (K = 16 each) into the TMEM accumulator and commits them to the chunk's stage
-// mbarrier; two stages alternate, so the next chunk's copies overlap this chunk's MMAs. The
-// epilogue reads the accumulator row by row (thread = row, tcgen05.ld.32x32b) and hands every
-// element (m, n, acc) to the layer's epilogue functor. Waits are bounded: on expiry the block
-// records MDG_STATUS_TIMEOUT, drains its MMAs, skips its epilogue and frees its TMEM.
-constexpr int kGemmThreads = 128;
-
-template <int BN>
-struct GemmShape {
-    static constexpr uint32_t a_bytes = 128 * 128;                    // [128 x 64] bf16
-    static constexpr uint32_t b_bytes = BN * 128;                     // [BN x 64] bf16
-    static constexpr uint32_t stage_bytes = a_bytes + b_bytes;
-    static constexpr uint32_t smem = 1024 + 2 * stage_bytes;          // alignment slack + two stages
-    static constexpr uint32_t tmem_cols = BN < 32 ? 32 : BN;
-};
-
-// Copies rows [row0, row0 + rows) x columns [k0, k0 + kw) (kw = 64 or 32) of a K-major bf16
-// matrix (leading dimension ld elements) into a swizzled [rows x 64] chunk at `dst`; columns
-// beyond kw are zero.
-__device__ __forceinline__ void load_chunk(uint32_t dst, const __nv_bfloat16* src, int ld, int row0, int rows, int k0,
-                                           int kw, uint8_t* dst_generic)
-{
-    const int pieces = kw / 8;
-    for (int i = threadIdx.x; i < rows * 8; i += kGemmThreads) {
-        const int r = i >> 3, k8 = i & 7;
-        const uint32_t off = (uint32_t)r * 128 + ((k8 ^ (r & 7)) << 4);
-        if (k8 < pieces) cp_async16(dst + off, src + (size_t)(row0 + r) * ld + k0 + k8 * 8);
-        else *reinterpret_cast<uint4*>(dst_generic + off) = make_uint4(0u, 0u, 0u, 0u);
-    }
-}
-
-template <int BN, class Epi>
-__global__ void __launch_bounds__(kGemmThreads) umma_gemm_kernel(const __nv_bfloat16* __restrict__ A, int lda,
-                                                                 const __nv_bfloat16* __restrict__ B, int ldb, int K,
-                                                                 int k_per_split, Epi epi, uint32_t* status)
-{
-    using S = GemmShape<BN>;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t bars[3];  // stage 0, stage 1: MMAs done with the stage; 2: accumulator done
-    __shared__ uint32_t s_tmem;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * 128, n0 = blockIdx.x * BN;
-    const int k_begin = blockIdx.z * k_per_split;
-    const int k_end = min(K, k_begin + k_per_split);
-    const uint32_t bar0 = smem_u32(&bars[0]);
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar0 + 8u * i));
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
-                     "r"(S::tmem_cols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = s_tmem;
-    const uint32_t idesc = idesc_bf16(128, BN);
-
-    bool ok = true;
-    int c = 0;  // chunks issued
-    for (int k0 = k_begin; k0 < k_end; k0 += 64, ++c) {
-        const int st = c & 1;
-        if (c >= 2) {  // the MMAs of chunk c - 2 have read this stage
-            const bool done = mbar_wait(bar0 + 8u * st, ((c - 2) >> 1) & 1, nullptr, status, kWaitLimit);
-            ok = __syncthreads_and(done);
-            if (!ok) break;
-        }
-        const int kw = min(64, k_end - k0);
-        uint8_t* sa = base + st * S::stage_bytes;
-        uint8_t* sb = sa + S::a_bytes;
-        load_chunk(smem_u32(sa), A, lda, m0, 128, k0, kw, sa);
-        load_chunk(smem_u32(sb), B, ldb, n0, BN, k0, kw, sb);
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                mma_bf16_ss(tmem, sw128_desc(smem_u32(sa) + kk * 32), sw128_desc(smem_u32(sb) + kk * 32), idesc,
-                            (c > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(bar0 + 8u * st);
-        }
-    }
-    // every MMA issued has completed before the accumulator is read or the TMEM freed
-    if (threadIdx.x == 0) mma_commit(bar0 + 16u);
-    const bool drained = mbar_wait(bar0 + 16u, 0, nullptr, status, kWaitLimit);
-    ok = __syncthreads_and(ok && drained && c > 0);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (ok) {
-        const int row = warp * 32 + lane;
-        const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
-        float loss = 0.f;
-#pragma unroll 1
-        for (int cc = 0; cc < BN; cc += 16) {
-            float v[16];
-            tmem_ld16(t_row + cc, v);
-            loss += epi.chunk(m0 + row, n0 + cc, v);
-        }
-        epi.finish(loss);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(S::tmem_cols));
-}
-
-__device__ __forceinline__ float silu_train(float z) { return z / (1.f + __expf(-z)); }
-__device__ __forceinline__ float silu_grad_train(float z)
-{
-    const float sg = 1.f / (1.f + __expf(-z));
-    return sg * (1.f + z * (1.f - sg));
-}
-
-// The epilogues take the 16 consecutive accumulator columns n0 .. n0 + 15 of row m (one
-// thread per row): row-major outputs are written 16 bytes at a time, transposed outputs one
-// element per thread, consecutive rows of a warp side by side.
-__device__ __forceinline__ void store_bf16x16(__nv_bfloat16* dst, const float v[16])
-{
-    uint32_t w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-        w[i] = *reinterpret_cast<const uint32_t*>(&p);
-    }
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-}
-__device__ __forceinline__ void store_f32x16(float* dst, const float v[16])
-{
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        reinterpret_cast<float4*>(dst)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-}
-__device__ __forceinline__ void load_f32x16(const float* src, float v[16])
-{
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 t = reinterpret_cast<const float4*>(src)[i];
-        v[4 * i] = t.x, v[4 * i + 1] = t.y, v[4 * i + 2] = t.z, v[4 * i + 3] = t.w;
-    }
-}
-
-// Hidden layer forward: z = acc + b[n] (FP32, kept for the backward pass), h = bf16(silu(z))
-// row-major and transposed (the transposed copy is the K-major operand of the weight gradient).
-struct TrainEpiHidden {
-    const float* bias;
-    float* z;
-    __nv_bfloat16* h;
-    __nv_bfloat16* hT;
-    int ld, ldT;
-    __device__ __forceinline__ float chunk(int m, int n0, const float acc[16]) const
-    {
-        float zz[16], hv[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            zz[i] = acc[i] + bias[n0 + i];
-            hv[i] = silu_train(zz[i]);
-        }
-        store_f32x16(z + (size_t)m * ld + n0, zz);
-        store_bf16x16(h + (size_t)m * ld + n0, hv);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) hT[(size_t)(n0 + i) * ldT + m] = __float2bfloat16_rn(hv[i]);
-        return 0.f;
-    }
-    __device__ __forceinline__ void finish(float) const {}
-};
-
-// Output layer forward with the MSE: y = acc + b[n]; on the n_valid used columns
-// dy = scale (y - t) (bf16, row-major and transposed) and loss += (y - t)^2 / (rows n_valid).
-struct TrainEpiOut {
-    const float* bias;
-    float* y;
-    const float* target;
-    __nv_bfloat16* dy;
-    __nv_bfloat16* dyT;
-    float* loss_acc;
-    int ld, ldT, n_valid;
-    float grad_scale, loss_scale;
-    __device__ __forceinline__ float chunk(int m, int n0, const float acc[16]) const
-    {
-        float yy[16], tt[16], g[16];
-        load_f32x16(target + (size_t)m * ld + n0, tt);
-        float loss = 0.f;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            yy[i] = acc[i] + bias[n0 + i];
-            const float d = n0 + i < n_valid ? yy[i] - tt[i] : 0.f;
-            g[i] = grad_scale * d;
-            loss += d * d * loss_scale;
-        }
-        store_f32x16(y + (size_t)m * ld + n0, yy);
-        store_bf16x16(dy + (size_t)m * ld + n0, g);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) dyT[(size_t)(n0 + i) * ldT + m] = __float2bfloat16_rn(g[i]);
-        return loss;
-    }
-    __device__ __forceinline__ void finish(float loss) const
-    {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(loss_acc, loss);
-    }
-};
-
-// Input gradient of a hidden layer: dz_prev = bf16(acc silu'(z_prev)), row-major and transposed.
-struct TrainEpiDx {
-    const float* zprev;
-    __nv_bfloat16* dz;
-    __nv_bfloat16* dzT;
-    int ld, ldT;
-    __device__ __forceinline__ float chunk(int m, int n0, const float acc[16]) const
-    {
-        float zp[16], g[16];
-        load_f32x16(zprev + (size_t)m * ld + n0, zp);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) g[i] = acc[i] * silu_grad_train(zp[i]);
-        store_bf16x16(dz + (size_t)m * ld + n0, g);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) dzT[(size_t)(n0 + i) * ldT + m] = __float2bfloat16_rn(g[i]);
-        return 0.f;
-    }
-    __device__ __forceinline__ void finish(float) const {}
-};
-
-// Weight gradient (split over K = the batch): g[m][n] (or g[n][m] when transposed) += acc,
-// four columns per vector reduction in the row-major case.
-struct TrainEpiGrad {
-    float* g;
-    int ld;
-    bool transpose;
-    __device__ __forceinline__ float chunk(int m, int n0, const float acc[16]) const
-    {
-        if (transpose) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) atomicAdd(g + (size_t)(n0 + i) * ld + m, acc[i]);
-        } else {
-            float4* row = reinterpret_cast<float4*>(g + (size_t)m * ld + n0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                atomicAdd(row + i, make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]));
-        }
-        return 0.f;
-    }
-    __device__ __forceinline__ void finish(float) const {}
-};
-
-// out[c][r] = in[r][c] for a [rows x cols] bf16 matrix (32 x 32 tiles through shared memory).
-__global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in,
-                                                             __nv_bfloat16* __restrict__ out, int rows, int cols)
-{
-    __shared__ __nv_bfloat16 tile[32][34];
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8)
-        if (r0 + i < rows && c0 + tx < cols) tile[i][tx] = in[(size_t)(r0 + i) * cols + c0 + tx];
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8)
-        if (c0 + i < cols && r0 + tx < rows) out[(size_t)(c0 + i) * rows + r0 + tx] = tile[tx][i];
-}
-
 // One thread per 16-byte piece (8 consecutive k of one row n) of every weight matrix.
 __global__ void build_image_kernel(const __nv_bfloat16* __restrict__ w16, MlpView w, uint8_t* __restrict__ img)
 {
@@ -1150,25 +697,6 @@ cudaError_t mlp_build_image(const MlpView& w, void* img, cudaStream_t s)
     return cudaGetLastError();
 }
 
-namespace {
-// cuTensorMapEncodeTiled, looked up through the runtime (no link against the driver library).
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_tiled()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-}  // namespace
-
 cudaError_t mlp_forward_umma_pairs(const MlpView& w, const void* img, const void* x, int B, float* y,
                                    uint32_t* status, int wait_limit, int spin_limit, cudaStream_t s,
                                    const MlpApply* apply)
@@ -1176,7 +704,6 @@ cudaError_t mlp_forward_umma_pairs(const MlpView& w, const void* img, const void
     if (B % kRows) return cudaErrorInvalidValue;
     const int n_tiles = B / kRows;
     if (n_tiles == 0) return cudaSuccess;
-    if (reinterpret_cast<uintptr_t>(x) % 16) return cudaErrorMisalignedAddress;  // TMA source
     static bool attr_done[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1191,18 +718,8 @@ cudaError_t mlp_forward_umma_pairs(const MlpView& w, const void* img, const void
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
-    const EncodeTiledFn encode = encode_tiled();
-    if (!encode) return cudaErrorNotSupported;
-    // the inputs [B x 64] bf16, row-major: boxes of one tile (128 rows x 128 bytes), 128-byte swizzle
     CUtensorMap xmap;
-    const cuuint64_t dims[2] = {MDG_MLP_IN_PAD, (cuuint64_t)B};
-    const cuuint64_t strides[1] = {MDG_MLP_IN_PAD * sizeof(__nv_bfloat16)};
-    const cuuint32_t box[2] = {MDG_MLP_IN_PAD, kRows};
-    const cuuint32_t elem_strides[2] = {1, 1};
-    if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), dims, strides, box, elem_strides,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
+    if ((e = input_map(&xmap, x, B)) != cudaSuccess) return e;
     int n_sm = 152;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int n_pairs = (n_tiles + 1) / 2;
@@ -1240,108 +757,6 @@ cudaError_t mlp_forward_umma(const MlpView& w, const void* img, const void* x, i
                                                       static_cast<const uint8_t*>(img), w.master, w, status,
                                                       wait_limit, spin_limit);
     return cudaGetLastError();
-}
-
-template <int BN, class Epi>
-static cudaError_t umma_gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N, int K,
-                             int splits, Epi epi, uint32_t* status, cudaStream_t s)
-{
-    if (M % 128 || N % BN || K % 32 || K <= 0 || splits < 1) return cudaErrorInvalidValue;
-    using S = GemmShape<BN>;
-    static bool attr_done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_done[dev]) {
-        e = cudaFuncSetAttribute(umma_gemm_kernel<BN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
-        if (e != cudaSuccess) return e;
-        attr_done[dev] = true;
-    }
-    // K per split: whole 64-wide chunks
-    const int chunks = (K + 63) / 64;
-    const int per = (chunks + splits - 1) / splits;
-    splits = (chunks + per - 1) / per;
-    dim3 grid(N / BN, M / 128, splits);
-    umma_gemm_kernel<BN, Epi><<<grid, kGemmThreads, S::smem, s>>>(reinterpret_cast<const __nv_bfloat16*>(A), lda,
-                                                                  reinterpret_cast<const __nv_bfloat16*>(B), ldb, K,
-                                                                  per * 64, epi, status);
-    return cudaGetLastError();
-}
-
-static cudaError_t transpose_bf16(const void* in, void* out, int rows, int cols, cudaStream_t s)
-{
-    dim3 grid((cols + 31) / 32, (rows + 31) / 32);
-    transpose_bf16_kernel<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(in), static_cast<__nv_bfloat16*>(out),
-                                               rows, cols);
-    return cudaGetLastError();
-}
-
-cudaError_t mlp_weights_transposed(const MlpView& w, void* wT, cudaStream_t s)
-{
-    // W2^T, W3^T [256 x 256] and W4^T [256 x 32] (the B operands of the input gradients)
-    const __nv_bfloat16* w16 = static_cast<const __nv_bfloat16*>(w.w16);
-    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(wT);
-    cudaError_t e = transpose_bf16(w16 + w.w_off[1], o, MDG_MLP_HIDDEN, MDG_MLP_HIDDEN, s);
-    if (e == cudaSuccess) e = transpose_bf16(w16 + w.w_off[2], o + MDG_MLP_HIDDEN * MDG_MLP_HIDDEN, MDG_MLP_HIDDEN,
-                                             MDG_MLP_HIDDEN, s);
-    if (e == cudaSuccess) e = transpose_bf16(w16 + w.w_off[3], o + 2 * MDG_MLP_HIDDEN * MDG_MLP_HIDDEN,
-                                             MDG_MLP_OUT_PAD, MDG_MLP_HIDDEN, s);
-    return e;
-}
-
-size_t mlp_weights_transposed_elems() { return 2 * MDG_MLP_HIDDEN * MDG_MLP_HIDDEN + MDG_MLP_HIDDEN * MDG_MLP_OUT_PAD; }
-
-cudaError_t mlp_grad_umma(const MlpView& w, const TrainBuffers& t, const void* x, int B, const float* target,
-                          float* loss_acc, float* grad, uint32_t* status, cudaStream_t s)
-{
-    const int H = MDG_MLP_HIDDEN, I = MDG_MLP_IN_PAD, O = MDG_MLP_OUT_PAD;
-    const __nv_bfloat16* w16 = static_cast<const __nv_bfloat16*>(w.w16);
-    const __nv_bfloat16* xin = static_cast<const __nv_bfloat16*>(x);
-    const __nv_bfloat16* wT = static_cast<const __nv_bfloat16*>(t.wT);
-    auto bf = [](void* p) { return static_cast<__nv_bfloat16*>(p); };
-    // the weight gradients are split over the batch and added up with atomics
-    const int splits = B / 256 > 0 ? B / 256 : 1;
-    cudaError_t e = cudaMemsetAsync(grad, 0, (size_t)MDG_MLP_PARAMS * 4, s);
-    if (e == cudaSuccess) e = transpose_bf16(x, t.xT, B, I, s);
-    // forward
-    const __nv_bfloat16* in = xin;
-    int fan_in = I;
-    for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
-        TrainEpiHidden ep{w.master + w.b_off[l], t.z[l], bf(t.h[l]), bf(t.hT[l]), H, B};
-        e = umma_gemm<128>(in, fan_in, w16 + w.w_off[l], fan_in, B, H, fan_in, 1, ep, status, s);
-        in = bf(t.h[l]);
-        fan_in = H;
-    }
-    if (e == cudaSuccess) {
-        TrainEpiOut eo{w.master + w.b_off[3], t.y, target, bf(t.dy), bf(t.dyT), loss_acc, O, B, MDG_MLP_OUT,
-                       2.f / ((float)B * MDG_MLP_OUT), 1.f / ((float)B * MDG_MLP_OUT)};
-        e = umma_gemm<32>(in, H, w16 + w.w_off[3], H, B, O, H, 1, eo, status, s);
-    }
-    // backward: output layer (dW4 as its transpose [256 x 32] = H3^T dY)
-    if (e == cudaSuccess) {
-        TrainEpiGrad eg{grad + w.w_off[3], H, true};
-        e = umma_gemm<32>(bf(t.hT[2]), B, bf(t.dyT), B, H, O, B, splits, eg, status, s);
-    }
-    if (e == cudaSuccess) e = mlp_bias_grad(t.dy, B, O, grad + w.b_off[3], s);
-    if (e == cudaSuccess) {  // dH3 = dY W4 (K = 32) -> dZ3
-        TrainEpiDx ex{t.z[2], bf(t.dz[2]), bf(t.dzT[2]), H, B};
-        e = umma_gemm<128>(bf(t.dy), O, wT + 2 * H * H, O, B, H, O, 1, ex, status, s);
-    }
-    // hidden layers l = 2, 1, 0 (weights W3, W2, W1)
-    for (int l = 2; l >= 0 && e == cudaSuccess; --l) {
-        const int fi = l == 0 ? I : H;
-        const __nv_bfloat16* inT = l == 0 ? bf(t.xT) : bf(t.hT[l - 1]);
-        TrainEpiGrad eg{grad + w.w_off[l], fi, false};
-        if (fi == H) e = umma_gemm<128>(bf(t.dzT[l]), B, inT, B, H, fi, B, splits, eg, status, s);
-        else e = umma_gemm<64>(bf(t.dzT[l]), B, inT, B, H, fi, B, splits, eg, status, s);
-        if (e == cudaSuccess) e = mlp_bias_grad(t.dz[l], B, H, grad + w.b_off[l], s);
-        if (e == cudaSuccess && l > 0) {  // dH_{l-1} = dZ_l W_l -> dZ_{l-1}
-            TrainEpiDx ex{t.z[l - 1], bf(t.dz[l - 1]), bf(t.dzT[l - 1]), H, B};
-            e = umma_gemm<128>(bf(t.dz[l]), H, wT + (size_t)(l - 1) * H * H, H, B, H, H, 1, ex, status, s);
-        }
-    }
-    return e;
 }
 
 }  // namespace mdg

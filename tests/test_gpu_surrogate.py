@@ -215,6 +215,34 @@ def test_gradients_and_loss_match_oracle(cuda, path, B):
     assert np.all(g[0][0][:, mdg.MLP_IN:] == 0)  # padded inputs get no gradient
 
 
+@pytest.mark.parametrize("B", [128, 384, 9856])
+def test_gradients_over_uneven_tile_shares(cuda, B):
+    """One tile, fewer tiles than shares, and 77 tiles in shares of 4 and 7 with the last ones
+    short or empty: the bounds of the weight-gradient kernel's split over the batch."""
+    test_gradients_and_loss_match_oracle(cuda, mdg.MLP_PATH_TCGEN05, B)
+
+
+def test_adam_refreshes_the_weight_image(cuda):
+    """The forward pass after an Adam step equals, bit for bit, that of a network created with
+    the updated parameters (whose image is built from their bf16 copies)."""
+    B = 256
+    m = mdg.MLP(B, _layers(21))
+    x = torch.as_tensor(_inputs(22, B), device=cuda).to(torch.bfloat16)
+    t = torch.full((B, mdg.MLP_OUT_PAD), 0.25, device=cuda)
+    for _ in range(2):
+        m.grad(x, t)
+        m.adam(1e-2)
+    fresh = mdg.MLP(B, m.params())
+    for path in (mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_TCGEN05_PAIRS):
+        ys = []
+        for net in (m, fresh):
+            net.set_path(path)
+            y = torch.empty((B, mdg.MLP_OUT_PAD), device=cuda)
+            net.forward(x, y)
+            ys.append(y)
+        assert torch.equal(*ys)
+
+
 def test_adam_matches_oracle(cuda):
     B = 128
     layers = _layers(6)

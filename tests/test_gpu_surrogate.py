@@ -587,3 +587,65 @@ def test_surrogate_step_composes_its_parts(cuda, trained, recipe):
         want[:, 3:7] /= np.linalg.norm(want[:, 3:7], axis=1, keepdims=True)
         got = sg.state13(state).double().cpu().numpy()
         assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(np.abs(want), 1.0)), np.abs(got - want).max()
+
+
+@pytest.mark.parametrize("N", [130, 1024, 1025, 40003, 600001])
+def test_fit_normalization_at_tile_edges(cuda, N):
+    """Row counts around the tiles' sizes and, at 600001, a sample stride of 2: statistics and rows
+    against numpy in float64, and the same result, bit for bit, from sets that are only 4-byte
+    aligned (the scalar copies). Tolerances: the statistics round to float32 once (6e-8; 1e-6 allows
+    the box edges' own rounding to move no row), targets take one subtraction and one division
+    (2e-7 of the largest term, at most 8 standard deviations about a mean of at most 2)."""
+    rng = np.random.default_rng(N)
+    raw = (rng.standard_normal((N, mdg.MLP_IN)) * np.linspace(0.1, 3, mdg.MLP_IN) + 2.0).astype(np.float32)
+    delta = rng.standard_normal((N, mdg.MLP_OUT)).astype(np.float32)
+    raw[:, 40] = 0.0
+    raw[N // 2, 3] = np.inf
+    delta[N - 1, 12] = np.nan
+    got = []
+    for shift in (0, 1):  # floats in front of each set
+        buf = [torch.zeros(a.size + shift, device=cuda) for a in (raw, delta)]
+        sets = []
+        for b, a in zip(buf, (raw, delta)):
+            b[shift:] = torch.as_tensor(a.reshape(-1), device=cuda)
+            sets.append(b[shift:].reshape(a.shape))
+        m = mdg.MLP(128)
+        x = torch.zeros((N, mdg.MLP_IN_PAD), dtype=torch.bfloat16, device=cuda)
+        t = torch.zeros((N, mdg.MLP_OUT_PAD), device=cuda)
+        got.append((m.fit_normalization(*sets, x, t), m.normalization(), x, t))
+    (counts, norm, x, t), (counts1, norm1, x1, t1) = got
+    assert counts == counts1 and all(np.array_equal(a, b) for a, b in zip(norm, norm1))
+    assert torch.equal(x, x1) and torch.equal(t, t1)
+    F = np.concatenate([raw, delta], 1).astype(np.float64)
+    F = F[np.isfinite(F).all(1)]
+    assert counts[0] == N - 2 == F.shape[0]
+    S = F[::max(1, F.shape[0] // 262144)]
+    qlo, qhi = np.quantile(S, float(np.float32(0.005)), axis=0), np.quantile(S, 1 - float(np.float32(0.005)), axis=0)
+    lo, hi = (qlo - 0.1 * (qhi - qlo)).astype(np.float32), (qhi + 0.1 * (qhi - qlo)).astype(np.float32)
+    K = F[((F >= lo) & (F <= hi)).all(1)]
+    mean, sd = K.mean(0), K.std(0, ddof=1)
+    sd[40] = 1.0
+    np.testing.assert_allclose(np.concatenate([norm[0], norm[2]]), mean, rtol=1e-6, atol=1e-7)
+    np.testing.assert_allclose(np.concatenate([norm[1], norm[3]]), sd, rtol=1e-6)
+    Z = (K - mean) / sd
+    Z = Z[(np.abs(Z[:, :mdg.MLP_IN]) <= 4.0).all(1) & (np.abs(Z[:, mdg.MLP_IN:]) <= 8.0).all(1)]
+    n = Z.shape[0] // 128 * 128
+    assert counts[1] == n
+    np.testing.assert_allclose(t[:n, :mdg.MLP_OUT].cpu().numpy(), Z[:n, mdg.MLP_IN:], rtol=1e-6, atol=3e-6)
+    # bf16: half an ulp (2^-9 relative) of the float32 value
+    np.testing.assert_allclose(x[:n, :mdg.MLP_IN].float().cpu().numpy(), Z[:n, :mdg.MLP_IN], rtol=2.0 ** -8, atol=1e-4)
+    assert not x[:n, mdg.MLP_IN:].any() and not t[:n, mdg.MLP_OUT:].any() and not x[n:].any() and not t[n:].any()
+
+
+def test_fit_normalization_without_usable_rows(cuda):
+    """No finite row, and a single one: refused, and the outputs stay as they were."""
+    m = mdg.MLP(128)
+    for finite in (0, 1):
+        raw = torch.full((300, mdg.MLP_IN), float("nan"), device=cuda)
+        delta = torch.zeros((300, mdg.MLP_OUT), device=cuda)
+        raw[:finite] = 1.0
+        x = torch.ones((300, mdg.MLP_IN_PAD), dtype=torch.bfloat16, device=cuda)
+        t = torch.ones((300, mdg.MLP_OUT_PAD), device=cuda)
+        with pytest.raises(mdg.MdgError):
+            m.fit_normalization(raw, delta, x, t)
+        assert torch.all(x == 1) and torch.all(t == 1)

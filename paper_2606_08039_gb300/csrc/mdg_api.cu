@@ -1043,6 +1043,7 @@ int mdg_render(mdg_handle h, const float* state, uint8_t* rgba, float* depth, in
     a.semi_a = (float)(h->cc.arm + h->cc.prop_radius);
     a.semi_c = (float)(0.3 * (h->cc.arm + h->cc.prop_radius));
     a.max_env = h->max_env;
+    a.vec = aligned16(rgba) && aligned16(depth) && aligned16(seg);
     a.status = h->d_status;
     cudaError_t e = mdg::launch_render(a, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "mdg_render: launch");

@@ -184,6 +184,7 @@ struct CamArgs {
     int* seg;                // [n][48 * 64] or null
     float semi_a, semi_c;    // the drones' ellipsoid semi-axes (a, a, c)
     int max_env;             // drones of the largest environment (shared-memory size)
+    int vec;                 // every output given is 16-byte aligned
     uint32_t* status;        // debug builds: MDG_STATUS_BOUNDS
 };
 cudaError_t launch_render(const CamArgs& a, cudaStream_t s);

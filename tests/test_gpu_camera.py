@@ -105,3 +105,52 @@ def test_optional_outputs_and_arguments(cuda):
     assert torch.equal(seg, seg2) and torch.equal(rgba, rgba3)
     L = mdg.lib()
     assert L.mdg_render(h._h, state.data_ptr(), rgba.data_ptr() + 1, None, None, None) == mdg.ERR_ARG
+
+
+@pytest.mark.parametrize("drones", [33, 70])
+def test_large_environments_match_oracle(cuda, drones):
+    """A block per camera: with tile masks (33 drones) and with rectangles per drone (70), on the
+    level lattice of the other recipes (tumbling cameras at this density see more than the 1% of
+    pixels that the check allows near a silhouette or a far checker edge)."""
+    sw = wl.full_aero(106, n_envs=1, drones=drones)
+    p, q, v, w = sw.p, sw.q, sw.v, sw.w
+    h = mdg.Handle([drones], [7])
+    state = mdg.pack_state(p, q, v, w, device=cuda)
+    frames = h.new_frames(cuda)
+    h.render(state, *frames)
+    torch.cuda.synchronize()
+    _check(h, oracle_arrays(state)[0], np.array([drones]), *frames, what=f"{drones} drones")
+
+
+def test_warp_and_block_forms_and_unaligned_outputs_agree(cuda):
+    """The same environments rendered by a warp per camera and, with a 33-drone environment in the
+    batch, by a block per camera; and into outputs that are only 4-byte aligned: bit for bit."""
+    sizes = np.array([1, 2, 4, 7, 32], np.int32)
+    n = int(sizes.sum())
+    p, q, v, w = wl.random_states(107, n + 33)
+    p[:3, 2] = [900.0, 3.0e4, -1.0]  # the horizon far away, and a camera below the ground
+    out = []
+    for extra in (0, 33):
+        dpe = np.concatenate([sizes, [extra]]).astype(np.int32)[:6 if extra else 5]
+        h = mdg.Handle(dpe, np.full(len(dpe), 7, np.uint32))
+        m = int(dpe.sum())
+        state = mdg.pack_state(p[:m], q[:m], v[:m], w[:m], device=cuda)
+        frames = h.new_frames(cuda)
+        h.render(state, *frames)
+        out.append([f[:n] for f in frames])
+        if not extra:
+            shp = (n, mdg.CAM_H, mdg.CAM_W)
+            px = n * mdg.CAM_H * mdg.CAM_W
+            raw = [torch.zeros(4 * px + 4, dtype=torch.uint8, device=cuda)[4:].reshape(shp + (4,)),
+                   torch.zeros(px + 1, device=cuda)[1:].reshape(shp),
+                   torch.zeros(px + 1, dtype=torch.int32, device=cuda)[1:].reshape(shp)]
+            h.render(state, *raw)
+            out.append(raw)
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert torch.equal(a, b)
+    rgba, depth, seg = (x.cpu().numpy() for x in out[0])
+    ground = seg == 0
+    assert np.all(np.isfinite(depth[ground])) and np.all(np.isinf(depth[seg == -1]))
+    greys = {tuple(c) for c in rgba[ground][:, :3]}
+    assert len(greys) == 2 and not ground[2].any()  # two greys; nothing seen from below

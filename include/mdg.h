@@ -310,7 +310,8 @@ int mdg_set_obs_bias(mdg_handle h, const float* obs_bias);
 
 /* Threads per block of the step kernels (a multiple of 32 in [32, 1024] and at least
  * the largest environment, rounded up to 32). Environments are packed whole into
- * blocks of at most this many drones. The default (chosen at creation) spreads the
+ * blocks of at most this many drones (randomized steps of uniform batches of up to 32
+ * drones per environment always take 64). The default (chosen at creation) spreads the
  * blocks evenly over the SMs; mdg_autotune picks by measurement. */
 int mdg_set_block_size(mdg_handle h, int32_t threads_per_block);
 int32_t mdg_get_block_size(mdg_handle h);

@@ -148,6 +148,7 @@ DevConsts make_dev_consts(const mdg_constants& c)
     d.inv_kf = (float)(1.0 / c.kf);
     d.hover_rpm = (float)sqrt(c.mass * c.g / (4.0 * c.kf));
     d.alloc_z = (float)(c.kf / c.km);
+    d.arm_f = d.kfm_f = 1.f;
     d.frame_p = c.frame == MDG_FRAME_P ? 1 : 0;
     d.rk4 = c.integrator == MDG_INTEGRATOR_RK4 ? 1 : 0;
     d.gnd_rotor = c.gnd_heights == MDG_GND_ROTOR ? 1 : 0;
@@ -764,7 +765,8 @@ int mdg_set_randomization(mdg_handle h, const float* env_params, float* motor, f
     ra.motor = reinterpret_cast<float4*>(motor);
     ra.hist = reinterpret_cast<float4*>(action_hist);
     ra.wind = reinterpret_cast<float4*>(wind_state);
-    ra.seed = seed;
+    ra.wind_key = mdg::stream_key(seed, mdg::kStreamWind);
+    ra.noise_key = mdg::stream_key(seed, mdg::kStreamObs);
     ra.depth = hist_depth;
     ra.obs_bias = h->dr ? h->rand_host.obs_bias : nullptr;  // an attached bias stays attached
     DeviceGuard dg(h->device);

@@ -45,6 +45,7 @@ struct DevConsts {
     int dsl;                          // 1: DSL controller (rate-limited setpoints; runtime-flag kernels)
     float sp_step_pos, sp_step_yaw;   // DSL setpoint limits per control period (rate x dt_ctrl)
     float rotor_x[4], rotor_y[4];     // rotor body positions (z = 0)
+    float arm_f, kfm_f;               // randomized models: the factors of L and of k_f / k_m
 };
 
 // A launch tile: whole environments packed into one thread block.
@@ -55,13 +56,31 @@ constexpr int kTileEnvMask = 0xffff;
 constexpr int kTileAnyDW = 1 << 30;      // some environment of the tile has downwash on
 constexpr int kTileWarpLocal = 1 << 29;  // every environment lies inside one warp
 
+// SplitMix64 (Steele, Lea, Flood, "Fast splittable pseudorandom number generators", OOPSLA 2014):
+// the output function of its counter-based form.
+__host__ __device__ inline unsigned long long splitmix64(unsigned long long z)
+{
+    z += 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+// The rounds that every draw of one seed and stream shares.
+__host__ __device__ inline unsigned long long stream_key(unsigned long long seed, unsigned long long stream)
+{
+    return splitmix64(splitmix64(seed) ^ stream);
+}
+constexpr unsigned long long kStreamWind = 21;  // random stream of the wind draws
+constexpr unsigned long long kStreamObs = 22;   // random stream of the observation noise
+
 // The buffers of mdg_set_randomization, kept in a small device allocation of the handle.
 struct RandArgs {
     const float* dr;          // [n_envs][MDG_DR_PARAMS] domain randomization and wind
     float4* motor;            // [n] rotor speeds (the motor lag's state)
     float4* hist;             // [depth][n] actions received (the latency's shift register)
     float4* wind;             // [n_envs][2] wind state
-    unsigned long long seed;  // of the wind draws
+    // the seed mixed with the streams of the wind draws and of the observation noise (stream_key)
+    unsigned long long wind_key, noise_key;
     int depth;
     const float4* obs_bias;   // [n][3] sticky per-episode observation bias (12 floats per drone), or null
 };

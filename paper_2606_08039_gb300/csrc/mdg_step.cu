@@ -11,6 +11,8 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <initializer_list>
+
 #include "mdg.h"
 #include "mdg_internal.cuh"
 
@@ -411,12 +413,16 @@ __device__ __forceinline__ float ground_increment(const Motor& m, float pz, floa
 {
     if ((kFlags == kFlagsRK4 || kFlags == kFlagsGndRotor || kFlags == kFlagsDR) && c.gnd_rotor) {
         const float R21 = 2.f * (qy * qz + qw * qx);
-        const float tx = c.alloc_xy * m.tau[0], ty = c.alloc_xy * m.tau[1], tz = c.alloc_z * m.tau[2];
+        // a randomized model keeps two factors across its substeps instead of ten products
+        const float fl = kFlags == kFlagsDR ? c.arm_f : 1.f;
+        const float axy = kFlags == kFlagsDR ? c.alloc_xy / fl : c.alloc_xy;
+        const float az = kFlags == kFlagsDR ? c.alloc_z * c.kfm_f : c.alloc_z;
+        const float tx = axy * m.tau[0], ty = axy * m.tau[1], tz = az * m.tau[2];
         float acc = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float f = 0.25f * (((m.T + c.mix_x[i] * tx) + c.mix_y[i] * ty) + ((i & 1) ? tz : -tz));
-            const float h = fmaxf(fmaf(R20, c.rotor_x[i], fmaf(R21, c.rotor_y[i], pz)), c.h_clip);
+            const float h = fmaxf(fmaf(R20, c.rotor_x[i] * fl, fmaf(R21, c.rotor_y[i] * fl, pz)), c.h_clip);
             acc = fmaf(f, rcp_approx(h * h), acc);
         }
         return c.gnd_k * acc;
@@ -659,20 +665,18 @@ __device__ __forceinline__ void write_knn(int4* __restrict__ nbr_idx, float* __r
 // strided 16-byte pieces, which the host link carries at a quarter of its rate and which
 // reach L2 as half-written sectors. Each warp stages its 32 consecutive rows in shared
 // memory (`stage`: 192 float4 of its own) and writes the contiguous span in 16-byte pieces,
-// lane by lane. `g` is the lane's output row; the active lanes form a prefix of the warp
+// lane by lane. `g` is the lane's output row, kin_row its KIN values; the active lanes form a prefix of the warp
 // and their rows are consecutive (lane 0's row + lane); every lane of the warp calls this.
 template <int kN>
 __device__ __forceinline__ void write_obs_staged(const StepArgs& a, float4* stage, bool active, long long g, int lane,
-                                                 long long env_first, int j, const Drone& d, const float rpm[4],
+                                                 long long env_first, int j, const Drone& d, const float4 kin_row[5],
                                                  const float4* env_pos, const float4* env_vel, int N_rt)
 {
     const int n_act = __popc(__ballot_sync(0xffffffffu, active));
     const long long g0 = __shfl_sync(0xffffffffu, g, 0);
     if (active) {
-        float4 v[5];
-        kin_values(d, rpm, v);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) stage[lane * 5 + k] = v[k];
+        for (int k = 0; k < 5; ++k) stage[lane * 5 + k] = kin_row[k];
     }
     __syncwarp();
     float4* kin = reinterpret_cast<float4*>(a.kin) + g0 * 5;
@@ -763,11 +767,11 @@ __device__ __forceinline__ void check_env(EnvSlot& e, int t, int n_drones, uint3
 
 
 // kN > 0: the batch is uniform with kN drones per environment (the compile-time variants
-// are launched only then), so the division below is by a constant.
+// are launched only then), so the division below is by a constant. t: the thread's place among
+// the tile's drones (threads beyond them get an empty slot); every thread of the block calls this.
 template <int kN = 0>
-__device__ __forceinline__ EnvSlot tile_env(const StepArgs& a, const TileInfo& ti, int* s_off, int* s_info)
+__device__ __forceinline__ EnvSlot tile_env(const StepArgs& a, const TileInfo& ti, int* s_off, int* s_info, int t)
 {
-    const int t = threadIdx.x;
     EnvSlot e = {0, 0, 0, 0, 0};
     if (a.uniform_N > 0) {
         if (t < ti.n_drones) {
@@ -781,9 +785,8 @@ __device__ __forceinline__ EnvSlot tile_env(const StepArgs& a, const TileInfo& t
         check_env(e, t, ti.n_drones, a.status);
         return e;
     }
-    const int B = blockDim.x;
-    for (int i = t; i <= ti.n_envs; i += B) s_off[i] = a.env_off[ti.first_env + i] - (int)ti.first_drone;
-    for (int i = t; i < ti.n_envs; i += B) {
+    for (int i = threadIdx.x; i <= ti.n_envs; i += blockDim.x) s_off[i] = a.env_off[ti.first_env + i] - (int)ti.first_drone;
+    for (int i = threadIdx.x; i < ti.n_envs; i += blockDim.x) {
         const int act = a.act_type == MDG_ACT_MIXED ? (int)a.env_act[ti.first_env + i] : a.act_type;
         s_info[i] = (int)a.env_flags[ti.first_env + i] | (act << 8);
     }
@@ -807,29 +810,15 @@ __device__ __forceinline__ EnvSlot tile_env(const StepArgs& a, const TileInfo& t
 
 // ---- domain randomization, motor lag, action latency and wind (kFlags == kFlagsDR) ----
 
-constexpr unsigned long long kStreamWind = 21;  // random stream of the wind draws
-
-// SplitMix64 (Steele, Lea, Flood, "Fast splittable pseudorandom number generators",
-// OOPSLA 2014): the output function of its counter-based form.
-__device__ __forceinline__ unsigned long long splitmix64(unsigned long long z)
-{
-    z += 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
 // U[0, 1) with 24 random bits (exact in float) for the counters (seed, stream, step,
 // index, comp), each mixed in by one SplitMix64 round. The rounds of (seed, stream, step,
-// index) form a prefix that all components of one draw share: counter_prefix mixes it once
-// and prefix_uniform adds the component's round (the same values as mixing all five).
-__device__ __forceinline__ unsigned long long counter_prefix(unsigned long long seed, unsigned long long stream,
-                                                             unsigned long long step, unsigned long long index)
+// index) form a prefix that all components of one draw share: stream_key mixes the first two,
+// counter_prefix the others, and prefix_uniform adds the component's round (the same values as
+// mixing all five).
+__device__ __forceinline__ unsigned long long counter_prefix(unsigned long long key, unsigned long long step,
+                                                             unsigned long long index)
 {
-    unsigned long long h = splitmix64(seed);
-    h = splitmix64(h ^ stream);
-    h = splitmix64(h ^ step);
-    return splitmix64(h ^ index);
+    return splitmix64(splitmix64(key ^ step) ^ index);
 }
 
 __device__ __forceinline__ float prefix_uniform(unsigned long long prefix, unsigned long long comp)
@@ -853,15 +842,10 @@ __device__ __forceinline__ DevConsts randomized_consts(const DevConsts& c, const
     }
     const float fl = row[MDG_DR_ARM], fkf = row[MDG_DR_KF], fkm = row[MDG_DR_KM];
     p.l_sqrt2 = c.l_sqrt2 * fl;
-    p.alloc_xy = c.alloc_xy / fl;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        p.rotor_x[i] = c.rotor_x[i] * fl;
-        p.rotor_y[i] = c.rotor_y[i] * fl;
-    }
+    p.arm_f = fl;
+    p.kfm_f = fkf / fkm;
     p.kf = c.kf * fkf;
     p.km = c.km * fkm;
-    p.alloc_z = c.alloc_z * (fkf / fkm);
     p.c_xy = c.c_xy * row[MDG_DR_CXY];
     p.c_z = c.c_z * row[MDG_DR_CZ];
     p.c_dz = p.c_z - p.c_xy;
@@ -873,18 +857,33 @@ __device__ __forceinline__ DevConsts randomized_consts(const DevConsts& c, const
 // Action latency: the action received enters the drone's shift register and the one
 // received `delay` control steps ago comes out (an empty register is first filled with
 // the action received).
-__device__ __forceinline__ float4 delayed_action(const StepArgs& a, long long g, const float4 act, int delay)
+__device__ __forceinline__ float4 delayed_action(const RandArgs& R, long long n, long long g, const float4 act, int delay)
 {
-    float4* h = a.rand->hist + g;
-    const int depth = a.rand->depth;
+    float4* h = R.hist + g;
+    const int depth = R.depth;
+    if (depth <= 4) {  // the register's rows in one round of loads
+        float4 v[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = k < depth ? h[k * n] : act;
+        const bool empty = isnan(v[0].x);
+        float4 out = act;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            const float4 u = empty ? act : v[k - 1];
+            if (k < depth) h[k * n] = u;
+            if (k == delay) out = u;
+        }
+        h[0] = act;
+        return out;
+    }
     if (isnan(h[0].x)) {
-        for (int k = 0; k < depth; ++k) h[k * a.n] = act;
+        for (int k = 0; k < depth; ++k) h[k * n] = act;
         return act;
     }
     float4 out = act;
     for (int k = depth - 1; k > 0; --k) {
-        const float4 v = h[(k - 1) * a.n];
-        h[k * a.n] = v;
+        const float4 v = h[(k - 1) * n];
+        h[k * n] = v;
         if (k == delay) out = v;
     }
     h[0] = act;
@@ -899,12 +898,12 @@ __device__ __forceinline__ float4 delayed_action(const StepArgs& a, long long g,
 // field starts a gust with the set probability, direction uniform on the sphere, force
 // A sin(pi s) while its phase s <= 1; SINUSOIDAL: A [sin wt, cos wt, 0.3 sin 2wt]. The gust
 // phase decides when a gust ends and advances in single precision.
-__device__ __forceinline__ void wind_step(const float* row, float4& s0, float4& s1, unsigned long long seed, int env,
+__device__ __forceinline__ void wind_step(const float* row, float4& s0, float4& s1, unsigned long long key, int env,
                                           float dt, float F[3], float vw[3])
 {
     const int model = (int)row[MDG_DR_WIND];
     const unsigned long long step = (unsigned long long)s1.w;
-    const unsigned long long wind_key = counter_prefix(seed, kStreamWind, step, env);
+    const unsigned long long wind_key = counter_prefix(key, step, env);
     F[0] = F[1] = F[2] = vw[0] = vw[1] = vw[2] = 0.f;
     if (model & MDG_WIND_CONSTANT) {
         vw[0] += row[MDG_DR_VWIND];
@@ -956,72 +955,131 @@ __device__ __forceinline__ void wind_step(const float* row, float4& s0, float4& 
     }
     if (model & MDG_WIND_SINUSOIDAL) {
         const float wt = row[MDG_DR_SIN_W] * ((float)step * dt), A = row[MDG_DR_SIN_A];
-        F[0] += A * sinf(wt);
-        F[1] += A * cosf(wt);
+        float sn, cs;
+        sincosf(wt, &sn, &cs);
+        F[0] += A * sn;
+        F[1] += A * cs;
         F[2] += A * 0.3f * sinf(2.f * wt);
     }
     s1.w = (float)(step + 1);
 }
 
-constexpr unsigned long long kStreamObs = 22;  // random stream of the observation noise
-
-// The KIN observation of d (RPMs a4) with the row's sensor noise: Gaussian (Box-Muller on the
-// counters (seed, kStreamObs, step, drone, 0..11)) of the row's sigmas on the position (0-2),
-// roll/pitch/yaw (3-5), velocity (6-8) and body rate (9-11), plus the drone's sticky
-// per-episode bias on the same channels when obs_bias ([n][12] as three float4) is given;
-// stored at kin_row[0..19].
-__device__ __forceinline__ void noisy_kin(float* kin_row, const Drone& d, const float a4[4], const float* row,
-                                          unsigned long long seed, unsigned long long step, long long g,
-                                          const float4* obs_bias)
+// The sensor noise of the row's sigmas and the drone's sticky bias (obs_bias: [n][3] float4, or
+// null), as an addition to the KIN row [p, q, rpy, v, w, a_prev]: Gaussian (Box-Muller on the
+// counters (seed, kStreamObs, step, drone, 0..11)) on the position (0-2), roll/pitch/yaw (3-5),
+// velocity (6-8) and body rate (9-11). `add(value, k)` receives channel k's noise, then its bias.
+// The pairs kFrom .. kTo - 1 of the six only (the bias with pair 0).
+template <int kFrom = 0, int kTo = 6, class Add>
+__device__ __forceinline__ void sensor_noise(const float* row, unsigned long long noise_key, unsigned long long step,
+                                             long long g, const float4* obs_bias, Add add)
 {
-    float4 v[5];
-    kin_values(d, a4, v);
     const float sp = row[MDG_DR_NOISE_P], sv = row[MDG_DR_NOISE_V], sr = row[MDG_DR_NOISE_RPY],
                 sw = row[MDG_DR_NOISE_W];
     if (sp > 0.f || sv > 0.f || sr > 0.f || sw > 0.f) {
-        float xi[12];
-        const unsigned long long key = counter_prefix(seed, kStreamObs, step, g);
+        const unsigned long long key = counter_prefix(noise_key, step, g);
+        const float sigma[4] = {sp, sr, sv, sw};
 #pragma unroll
-        for (int m = 0; m < 6; ++m) {
+        for (int m = kFrom; m < kTo; ++m) {
             const float u1 = 1.f - prefix_uniform(key, 2 * m);
             const float u2 = prefix_uniform(key, 2 * m + 1);
             const float r = sqrtf(-2.f * logf(u1));
             float sn, cs;
             sincospif(2.f * u2, &sn, &cs);  // sin and cos of 2 pi u2
-            xi[2 * m] = r * cs;
-            xi[2 * m + 1] = r * sn;
+            add(sigma[(2 * m) / 3] * (r * cs), 2 * m);
+            add(sigma[(2 * m + 1) / 3] * (r * sn), 2 * m + 1);
         }
-        v[0].x += sp * xi[0];
-        v[0].y += sp * xi[1];
-        v[0].z += sp * xi[2];
-        v[1].w += sr * xi[3];
-        v[2].x += sr * xi[4];
-        v[2].y += sr * xi[5];
-        v[2].z += sv * xi[6];
-        v[2].w += sv * xi[7];
-        v[3].x += sv * xi[8];
-        v[3].y += sw * xi[9];
-        v[3].z += sw * xi[10];
-        v[3].w += sw * xi[11];
     }
-    if (obs_bias) {  // [p (3), rpy (3), v (3), w (3)] as (p.xyz, roll) (pitch, yaw, v.xy) (v.z, w.xyz)
+    if (kFrom == 0 && obs_bias) {  // [p (3), rpy (3), v (3), w (3)]
         const float4 b0 = obs_bias[3 * g], b1 = obs_bias[3 * g + 1], b2 = obs_bias[3 * g + 2];
-        v[0].x += b0.x;
-        v[0].y += b0.y;
-        v[0].z += b0.z;
-        v[1].w += b0.w;
-        v[2].x += b1.x;
-        v[2].y += b1.y;
-        v[2].z += b1.z;
-        v[2].w += b1.w;
-        v[3].x += b2.x;
-        v[3].y += b2.y;
-        v[3].z += b2.z;
-        v[3].w += b2.w;
+        const float b[12] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w, b2.x, b2.y, b2.z, b2.w};
+#pragma unroll
+        for (int k = 0; k < 12; ++k) add(b[k], k);
     }
+}
+
+// The place of noise channel k in a KIN row [p (3), q (4), rpy (3), v (3), w (3), a_prev (4)].
+__device__ __forceinline__ constexpr int kin_channel(int k) { return k < 3 ? k : k + 4; }
+
+// KIN row of d (RPMs a4) with its noise and bias, as five float4.
+__device__ __forceinline__ void noisy_kin_values(const Drone& d, const float a4[4], const float* row,
+                                                 unsigned long long noise_key, unsigned long long step, long long g,
+                                                 const float4* obs_bias, float4 o[5])
+{
+    float4 v[5];
+    kin_values(d, a4, v);
+    float k[20];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) k[4 * i] = v[i].x, k[4 * i + 1] = v[i].y, k[4 * i + 2] = v[i].z, k[4 * i + 3] = v[i].w;
+    sensor_noise(row, noise_key, step, g, obs_bias, [&k](float x, int c) { k[kin_channel(c)] += x; });
+#pragma unroll
+    for (int i = 0; i < 5; ++i) o[i] = make_float4(k[4 * i], k[4 * i + 1], k[4 * i + 2], k[4 * i + 3]);
+}
+
+// The same, stored at kin_row[0..19].
+__device__ __forceinline__ void noisy_kin(float* kin_row, const Drone& d, const float a4[4], const float* row,
+                                          unsigned long long noise_key, unsigned long long step, long long g,
+                                          const float4* obs_bias)
+{
+    float4 v[5];
+    noisy_kin_values(d, a4, row, noise_key, step, g, obs_bias, v);
     float4* o = reinterpret_cast<float4*>(kin_row);
 #pragma unroll
     for (int k = 0; k < 5; ++k) o[k] = v[k];
+}
+
+// An environment's randomization row in registers: ten 16-byte loads (those of values that the
+// caller does not use are dropped).
+__device__ __forceinline__ void load_row(const float* dr, int env, float r[MDG_DR_PARAMS])
+{
+    const float4* p = reinterpret_cast<const float4*>(dr + (long long)env * MDG_DR_PARAMS);
+#pragma unroll
+    for (int i = 0; i < MDG_DR_PARAMS / 4; ++i) {
+        const float4 v = __ldg(p + i);
+        r[4 * i] = v.x, r[4 * i + 1] = v.y, r[4 * i + 2] = v.z, r[4 * i + 3] = v.w;
+    }
+}
+
+// What each drone needs of its row for the substeps: its motors' commands (RPM times bias, saturated
+// at MAX_RPM times the factor), the lag's decay over a substep, and the drag from the wind vw.
+__device__ __forceinline__ void motor_commands(const float* row, const float rpm[4], const DevConsts& c, float cmd[4],
+                                               float& lag)
+{
+    const float sat = c.max_rpm * row[MDG_DR_MAXRPM];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cmd[i] = fminf(rpm[i] * row[MDG_DR_BIAS + i], sat);
+    const float tau = row[MDG_DR_TAU];
+    lag = tau > 0.f ? expf(-c.dt_sim / tau) : 0.f;
+}
+__device__ __forceinline__ void wind_drag(const float* row, const float vw[3], const Drone& d, float F[3])
+{
+    const int model = (int)row[MDG_DR_WIND];
+    if (model & (MDG_WIND_CONSTANT | MDG_WIND_DRYDEN)) {
+        const float vr[3] = {vw[0] - d.v[0], vw[1] - d.v[1], vw[2] - d.v[2]};
+        const float k = row[MDG_DR_KDRAG] * sqrtf(vr[0] * vr[0] + vr[1] * vr[1] + vr[2] * vr[2]);
+        F[0] += k * vr[0];
+        F[1] += k * vr[1];
+        F[2] += k * vr[2];
+    }
+}
+__device__ __forceinline__ void start_motors(float4& ms, const float cmd[4])
+{
+    if (isnan(ms.x)) ms.x = cmd[0];
+    if (isnan(ms.y)) ms.y = cmd[1];
+    if (isnan(ms.z)) ms.z = cmd[2];
+    if (isnan(ms.w)) ms.w = cmd[3];
+}
+// One substep under the lag: n <- c + (n - c) exp(-dt/tau), then the randomized model.
+template <int kN>
+__device__ __forceinline__ void randomized_substep(Drone& d, float4& ms, const float cmd[4], float lag, int flags,
+                                                   const float4* env_pos, int N, int jl, const DevConsts& pc,
+                                                   const float3 fe)
+{
+    ms.x = cmd[0] + (ms.x - cmd[0]) * lag;
+    ms.y = cmd[1] + (ms.y - cmd[1]) * lag;
+    ms.z = cmd[2] + (ms.z - cmd[2]) * lag;
+    ms.w = cmd[3] + (ms.w - cmd[3]) * lag;
+    const float n[4] = {ms.x, ms.y, ms.z, ms.w};
+    substep<kFlagsDR, kN>(d, motor(n, pc), flags, env_pos, N, jl, pc, fe);
 }
 
 constexpr unsigned long long kStreamInit = 23;  // random stream of the per-episode initial states
@@ -1038,7 +1096,7 @@ __global__ void __launch_bounds__(256) reset_kernel(const ResetArgs r)
 {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= r.n) return;
-    const unsigned long long key = counter_prefix(r.seed, kStreamInit, r.episode, (unsigned long long)g);
+    const unsigned long long key = counter_prefix(stream_key(r.seed, kStreamInit), r.episode, (unsigned long long)g);
     float u[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) u[k] = 2.f * prefix_uniform(key, k) - 1.f;
@@ -1062,7 +1120,7 @@ __global__ void __launch_bounds__(256) reset_kernel(const ResetArgs r)
     S[4 * r.n + g] = make_float4(0.f, 0.f, 0.f, 0.f);
     S[5 * r.n + g] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r.obs_bias) {
-        const unsigned long long bkey = counter_prefix(r.seed, kStreamBias, r.episode, (unsigned long long)g);
+        const unsigned long long bkey = counter_prefix(stream_key(r.seed, kStreamBias), r.episode, (unsigned long long)g);
         float b[12];
 #pragma unroll
         for (int m = 0; m < 6; ++m) {
@@ -1099,7 +1157,6 @@ __device__ __forceinline__ void randomized_substeps(const StepArgs& a, Drone& d,
                                                     const float a_pre[4], bool& delayed, unsigned long long& step)
 {
     const RandArgs& R = *a.rand;
-    const float* row = R.dr + (long long)env.id * MDG_DR_PARAMS;
     __syncthreads();  // the previous control step's wind state is stored
     float4 s0 = {}, s1 = {}, ms = {};
     float cmd[4] = {0.f, 0.f, 0.f, 0.f}, lag = 0.f;
@@ -1108,33 +1165,21 @@ __device__ __forceinline__ void randomized_substeps(const StepArgs& a, Drone& d,
     delayed = false;
     step = 0;
     if (active) {
+        float row[MDG_DR_PARAMS];
+        load_row(R.dr, env.id, row);
         s0 = R.wind[2LL * env.id];
         s1 = R.wind[2LL * env.id + 1];
         step = (unsigned long long)s1.w;
         delayed = row[MDG_DR_OBS_DELAY] == 1.f;
-        if (kin_row && delayed) noisy_kin(kin_row, d, a_pre, row, R.seed, step, g, R.obs_bias);
+        if (kin_row && delayed) noisy_kin(kin_row, d, a_pre, row, R.noise_key, step, g, R.obs_bias);
         float Fd[3], vw[3];
-        wind_step(row, s0, s1, R.seed, env.id, a.c.dt_ctrl, Fd, vw);
-        const int model = (int)row[MDG_DR_WIND];
-        if (model & (MDG_WIND_CONSTANT | MDG_WIND_DRYDEN)) {
-            const float vr[3] = {vw[0] - d.v[0], vw[1] - d.v[1], vw[2] - d.v[2]};
-            const float k = row[MDG_DR_KDRAG] * sqrtf(vr[0] * vr[0] + vr[1] * vr[1] + vr[2] * vr[2]);
-            Fd[0] += k * vr[0];
-            Fd[1] += k * vr[1];
-            Fd[2] += k * vr[2];
-        }
+        wind_step(row, s0, s1, R.wind_key, env.id, a.c.dt_ctrl, Fd, vw);
+        wind_drag(row, vw, d, Fd);
         fe = make_float3(Fd[0], Fd[1], Fd[2]);
         pc = randomized_consts(a.c, row);
-        const float sat = a.c.max_rpm * row[MDG_DR_MAXRPM];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) cmd[i] = fminf(rpm[i] * row[MDG_DR_BIAS + i], sat);
-        const float tau = row[MDG_DR_TAU];
-        lag = tau > 0.f ? expf(-a.c.dt_sim / tau) : 0.f;
+        motor_commands(row, rpm, a.c, cmd, lag);
         ms = R.motor[g];
-        if (isnan(ms.x)) ms.x = cmd[0];
-        if (isnan(ms.y)) ms.y = cmd[1];
-        if (isnan(ms.z)) ms.z = cmd[2];
-        if (isnan(ms.w)) ms.w = cmd[3];
+        start_motors(ms, cmd);
     }
     __syncthreads();  // every drone has read the wind state
     if (active && t == env.ls) {
@@ -1148,14 +1193,7 @@ __device__ __forceinline__ void randomized_substeps(const StepArgs& a, Drone& d,
             if (warp_local) __syncwarp();
             else __syncthreads();
         }
-        if (active) {
-            ms.x = cmd[0] + (ms.x - cmd[0]) * lag;
-            ms.y = cmd[1] + (ms.y - cmd[1]) * lag;
-            ms.z = cmd[2] + (ms.z - cmd[2]) * lag;
-            ms.w = cmd[3] + (ms.w - cmd[3]) * lag;
-            const float n[4] = {ms.x, ms.y, ms.z, ms.w};
-            substep<kFlagsDR, kN>(d, motor(n, pc), env.flags, buf + env.ls, env.N, t - env.ls, pc, fe);
-        }
+        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf + env.ls, env.N, t - env.ls, pc, fe);
     }
     if (active) R.motor[g] = ms;
 }
@@ -1308,7 +1346,7 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
         if (a.act_type != MDG_ACT_RPM) s4 = a.state[4 * a.n + g];
         act = a.action[g];
     }
-    const EnvSlot env = tile_env<kN>(a, tile, s_off, s_info);
+    const EnvSlot env = tile_env<kN>(a, tile, s_off, s_info, t);
     const bool is_pid = env.act == MDG_ACT_PID;
     const bool loops = is_pid || (runtime_variant(kFlags) && uses_loops(env.act));
 
@@ -1320,7 +1358,7 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
     unsigned long long obs_step = 0;
     if (active) {
         if constexpr (kFlags == kFlagsDR) {  // action latency
-            act = delayed_action(a, g, act, (int)a.rand->dr[(long long)env.id * MDG_DR_PARAMS + MDG_DR_DELAY]);
+            act = delayed_action(*a.rand, a.n, g, act, (int)a.rand->dr[(long long)env.id * MDG_DR_PARAMS + MDG_DR_DELAY]);
             if (kObs) {
                 const float4 p5 = a.state[5 * a.n + g];
                 a_pre[0] = p5.x, a_pre[1] = p5.y, a_pre[2] = p5.z, a_pre[3] = p5.w;
@@ -1386,17 +1424,222 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
         if (kFlags != kFlagsDR || a.obs_host) {
             float4* stage = reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + obs_stage_offset(B)) +
                             (t >> 5) * 192;
-            write_obs_staged<kN>(a, stage, active, g, t & 31, tile.first_drone + env.ls, t - env.ls, d, rpm,
+            float4 kin[5] = {};
+            if (active) kin_values(d, rpm, kin);
+            write_obs_staged<kN>(a, stage, active, g, t & 31, tile.first_drone + env.ls, t - env.ls, d, kin,
                                  pb + env.ls, s_vel + env.ls, env.N);
         } else if (active) {
             if constexpr (kFlags == kFlagsDR) {  // sensor noise; delayed ones were written at the start
                 if (!delayed)
-                    noisy_kin(a.kin + 20 * g, d, rpm, a.rand->dr + (long long)env.id * MDG_DR_PARAMS, a.rand->seed,
-                              obs_step, g, a.rand->obs_bias);
+                    noisy_kin(a.kin + 20 * g, d, rpm, a.rand->dr + (long long)env.id * MDG_DR_PARAMS,
+                              a.rand->noise_key, obs_step, g, a.rand->obs_bias);
             }
             write_knn<kN>(a.nbr_idx, a.nbr_rel, g, tile.first_drone + env.ls, t - env.ls, d, pb + env.ls,
                           s_vel + env.ls, env.N);
         }
+    }
+}
+
+// ---- the control step under domain randomization, uniform batches of up to 32 drones ----
+//
+// The randomized step draws 7 wind uniforms per environment and 12 normals per drone beside the
+// dynamics. Drawn by the drones' own threads (step_kernel) they make one chain of ~4900
+// instructions per warp, with too few warps to hide it: 13.5 an SM on the 65,536-drone swarm, issue
+// slots 41% busy. Here a block holds 64 drones in two warps and a third warp that draws: first the
+// wind, one lane per environment instead of one per drone, while the drones' threads run the
+// controller; then four of the six pairs of sensor noise, while they run the substeps (with all six
+// it finishes last, with three the drones do: 115, 113 and 113 us a pass of 8 steps). The drones'
+// threads wait for it at two named barriers. The drawing warp also starts the KIN row of a drone
+// whose observation is delayed: it reports the step's start, which is in memory until the second
+// barrier. 80 registers, so that the swarm's 1024 blocks are resident at once. 8 steps of
+// 16384 x 4: 146 -> 114 us; 64 x 1: 102 -> 74; 65536 x 4: 518 -> 435. Above 32 drones the pair loops
+// outweigh the draws and want the registers (1024 x 64: 310 us in step_kernel, 338 so).
+constexpr int kDrawDrones = 64;  // drones of a block
+constexpr int kDrawPairs = 4;    // of the noise's six pairs: the drones' threads draw the other two
+constexpr int kBarWind = 1, kBarNoise = 2, kBarDrones = 3;
+__device__ __forceinline__ void named_sync(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Per environment of the block: its wind's force F (3) and velocity vw (3), step, delayed.
+struct DrawnWind {
+    float v[8];
+};
+
+// The drawing warp.
+template <bool kObs, int kN>
+__device__ __forceinline__ void draw_wind_and_noise(const StepArgs& a, const RandArgs& R, const TileInfo& tile,
+                                                    DrawnWind* s_wind, float4* s_row)
+{
+    const int lane = threadIdx.x & 31;
+    for (int e = lane; e < tile.n_envs; e += 32) {
+        const int id = tile.first_env + e;
+        float row[MDG_DR_PARAMS];
+        load_row(R.dr, id, row);
+        float4 s0 = R.wind[2LL * id], s1 = R.wind[2LL * id + 1];
+        float* w = s_wind[e].v;
+        w[6] = s1.w;
+        w[7] = row[MDG_DR_OBS_DELAY];
+        float F[3], vw[3];
+        wind_step(row, s0, s1, R.wind_key, id, a.c.dt_ctrl, F, vw);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) w[r] = F[r], w[3 + r] = vw[r];
+        R.wind[2LL * id] = s0;
+        R.wind[2LL * id + 1] = s1;
+    }
+    named_arrive(kBarWind, kDrawDrones + 32);
+    if constexpr (!kObs) return;
+    __syncwarp();
+    for (int t = lane; t < tile.n_drones; t += 32) {
+        const int e = t / (kN > 0 ? kN : a.uniform_N);
+        const long long g = tile.first_drone + t;
+        float row[MDG_DR_PARAMS];
+        load_row(R.dr, tile.first_env + e, row);
+        float4 v[5] = {};
+        if (s_wind[e].v[7] == 1.f) {
+            Drone d;
+            load_state(a.state, a.n, g, d, false);
+            const float4 p5 = a.state[5 * a.n + g];
+            const float a_pre[4] = {p5.x, p5.y, p5.z, p5.w};
+            kin_values(d, a_pre, v);
+        }
+        float k[20];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) k[4 * i] = v[i].x, k[4 * i + 1] = v[i].y, k[4 * i + 2] = v[i].z, k[4 * i + 3] = v[i].w;
+        sensor_noise<0, kDrawPairs>(row, R.noise_key, (unsigned long long)s_wind[e].v[6], g, R.obs_bias,
+                                    [&k](float x, int c) { k[kin_channel(c)] += x; });
+#pragma unroll
+        for (int i = 0; i < 5; ++i) s_row[5 * t + i] = make_float4(k[4 * i], k[4 * i + 1], k[4 * i + 2], k[4 * i + 3]);
+    }
+    named_arrive(kBarNoise, kDrawDrones + 32);
+}
+
+template <bool kObs, int kN>
+__global__ void __launch_bounds__(kDrawDrones + 32, 7) randomized_step_kernel(const StepArgs a)
+{
+    constexpr int B = kDrawDrones;
+    __shared__ float4 s_pos[2][B], s_vel[B];
+    __shared__ float4 s_stage[kObs ? B / 32 * 192 : 1], s_row[kObs ? 5 * B : 1];
+    __shared__ DrawnWind s_wind[B];
+
+    grid_wait();
+    const TileInfo tile = get_tile(a);
+    const int t = threadIdx.x;
+    const bool active = t < tile.n_drones;  // at most B: the drawing warp has none
+    const long long g = tile.first_drone + t;
+    const RandArgs R = *a.rand;
+    if (t >= B) {
+        draw_wind_and_noise<kObs, kN>(a, R, tile, s_wind, s_row);
+        return;
+    }
+    float4 s0 = {}, s1 = {}, s2 = {}, s3 = {}, s4 = {}, act = {}, ms = {};
+    if (active) {
+        s0 = a.state[g];
+        s1 = a.state[a.n + g];
+        s2 = a.state[2 * a.n + g];
+        s3 = a.state[3 * a.n + g];
+        if (a.act_type != MDG_ACT_RPM) s4 = a.state[4 * a.n + g];
+        act = a.action[g];
+        ms = R.motor[g];
+    }
+    const EnvSlot env = tile_env<kN>(a, tile, nullptr, nullptr, t);  // uniform: no tables
+    const DrawnWind& wind = s_wind[active ? env.id - tile.first_env : 0];
+    const bool loops = uses_loops(env.act);
+    const bool tile_dw = (tile.bits & kTileAnyDW) != 0;
+    const bool warp_local = (tile.bits & kTileWarpLocal) != 0;
+    auto drones_sync = [&]() {
+        if (warp_local) __syncwarp();
+        else named_sync(kBarDrones, B);
+    };
+    Drone d;
+    unpack_state(s0, s1, s2, s3, s4, d);
+    float row[MDG_DR_PARAMS];
+    float rpm[4] = {0.f, 0.f, 0.f, 0.f}, cmd[4] = {0.f, 0.f, 0.f, 0.f}, lag = 0.f;
+    DevConsts pc = a.c;
+    if (active) {
+        load_row(R.dr, env.id, row);
+        act = delayed_action(R, a.n, g, act, (int)row[MDG_DR_DELAY]);
+        if (env.act >= MDG_ACT_RPM_NORM) {
+            ext_action_rpm(d, act, env.act, a.c, rpm);
+        } else if (env.act == MDG_ACT_PID) {
+            float ep[3], ye;
+            const float4 wp = a.c.dsl ? dsl_setpoint(d, act, a.setpoints + g, a.c) : act;
+            pid(d, wp, a.c, rpm, ep, ye);
+        } else {
+            rpm[0] = fminf(a.c.max_rpm, fmaxf(0.f, act.x));
+            rpm[1] = fminf(a.c.max_rpm, fmaxf(0.f, act.y));
+            rpm[2] = fminf(a.c.max_rpm, fmaxf(0.f, act.z));
+            rpm[3] = fminf(a.c.max_rpm, fmaxf(0.f, act.w));
+        }
+        motor_commands(row, rpm, a.c, cmd, lag);
+        start_motors(ms, cmd);
+        pc = randomized_consts(a.c, row);
+    }
+    named_sync(kBarWind, B + 32);
+    float3 fe = {};
+    if (active) {
+        float F[3] = {wind.v[0], wind.v[1], wind.v[2]};
+        const float vw[3] = {wind.v[3], wind.v[4], wind.v[5]};
+        wind_drag(row, vw, d, F);
+        fe = make_float3(F[0], F[1], F[2]);
+    }
+    for (int s = 0; s < a.n_sub; ++s) {
+        float4* buf = s_pos[s & 1];
+        if (tile_dw) {
+            buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+            drones_sync();
+        }
+        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf + env.ls, env.N, t - env.ls, pc, fe);
+    }
+    float own[2 * (6 - kDrawPairs)] = {};  // the noise of the last channels
+    if constexpr (kObs) {
+        if (active) {
+            float sig[MDG_DR_PARAMS];
+            load_row(R.dr, env.id, sig);
+            sensor_noise<kDrawPairs, 6>(sig, R.noise_key, (unsigned long long)wind.v[6], g, nullptr,
+                                        [&own](float x, int c) { own[c - 2 * kDrawPairs] = x; });
+        }
+        named_sync(kBarNoise, B + 32);  // the state of the step's start has been read
+    }
+    bool bad = false;
+    if (active) {
+        R.motor[g] = ms;
+        store_state(a.state, a.n, g, d, loops);
+        a.state[5 * a.n + g] = make_float4(rpm[0], rpm[1], rpm[2], rpm[3]);
+        bad = !finite_state(d);
+    }
+    const unsigned bad_mask = __ballot_sync(0xffffffffu, bad);
+    if (bad_mask && (t & 31) == 0) {
+        atomicOr(a.status, MDG_STATUS_NONFINITE);
+        atomicMin(a.status + 1, (unsigned)(g + __ffs(bad_mask) - 1));
+    }
+    if constexpr (kObs) {
+        float4* pb = s_pos[a.n_sub & 1];  // not the buffer the last substep read
+        pb[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+        s_vel[t] = make_float4(d.v[0], d.v[1], d.v[2], 0.f);
+        float4 v[5] = {};
+        if (active) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) v[k] = s_row[5 * t + k];
+            if (wind.v[7] != 1.f) {  // not delayed: the noise alone is there
+                float4 kin[5];
+                kin_values(d, rpm, kin);
+#pragma unroll
+                for (int k = 0; k < 5; ++k)
+                    v[k] = make_float4(kin[k].x + v[k].x, kin[k].y + v[k].y, kin[k].z + v[k].z, kin[k].w + v[k].w);
+            }
+            float* k = reinterpret_cast<float*>(v);
+#pragma unroll
+            for (int c = 2 * kDrawPairs; c < 12; ++c) k[kin_channel(c)] += own[c - 2 * kDrawPairs];
+        }
+        drones_sync();
+        write_obs_staged<kN>(a, s_stage + (t >> 5) * 192, active, g, t & 31, tile.first_drone + env.ls, t - env.ls, d, v,
+                             pb + env.ls, s_vel + env.ls, env.N);
     }
 }
 
@@ -1545,7 +1788,7 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
             if (active && k + 1 < r.K) next = a.action[(k + 1) * r.action_stride + g];
             if (active) {
                 if constexpr (kFlags == kFlagsDR)  // action latency
-                    act = delayed_action(a, g, act, (int)a.rand->dr[(long long)env.id * MDG_DR_PARAMS + MDG_DR_DELAY]);
+                    act = delayed_action(*a.rand, a.n, g, act, (int)a.rand->dr[(long long)env.id * MDG_DR_PARAMS + MDG_DR_DELAY]);
                 if (runtime_variant(kFlags) && env.act >= MDG_ACT_RPM_NORM) {
                     ext_action_rpm(d, act, env.act, a.c, rpm);
                 } else if (is_pid) {
@@ -1594,7 +1837,7 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
                     if constexpr (kFlags == kFlagsDR) {  // sensor noise; delayed ones were written at the start
                         if (!delayed)
                             noisy_kin(a.kin + 20 * (o + g), d, rpm, a.rand->dr + (long long)env.id * MDG_DR_PARAMS,
-                                      a.rand->seed, obs_step, g, a.rand->obs_bias);
+                                      a.rand->noise_key, obs_step, g, a.rand->obs_bias);
                     } else {
                         rpy_of(d.q, rpy_c[0], rpy_c[1], rpy_c[2]);
                         have_rpy = true;
@@ -1643,7 +1886,7 @@ __global__ void __launch_bounds__(1024) obs_kernel(const StepArgs a)
         load_state(a.state, a.n, g, d, false);
         ap = a.state[5 * a.n + g];
     }
-    const EnvSlot env = tile_env(a, tile, s_off, s_info);
+    const EnvSlot env = tile_env(a, tile, s_off, s_info, t);
     s_pos[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
     s_vel[t] = make_float4(d.v[0], d.v[1], d.v[2], 0.f);
     __syncthreads();
@@ -1689,7 +1932,7 @@ __global__ void __launch_bounds__(1024) features_kernel(const SurrogateArgs sa)
         load_state(a.state, a.n, g, d, false);
         r4 = sa.rpm[g];
     }
-    const EnvSlot env = tile_env(a, tile, s_off, s_info);
+    const EnvSlot env = tile_env(a, tile, s_off, s_info, t);
     s_pos[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
     s_vel[t] = make_float4(d.v[0], d.v[1], d.v[2], 0.f);
     __syncthreads();
@@ -1731,7 +1974,7 @@ __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const Surrogate
         if (a.act_type != MDG_ACT_RPM) s4 = a.state[4 * a.n + g];
         act = a.action[g];
     }
-    const EnvSlot env = tile_env(a, tile, s_off, s_info);
+    const EnvSlot env = tile_env(a, tile, s_off, s_info, t);
     Drone d;
     unpack_state(s0, s1, s2, s3, s4, d);
     float rpm[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1966,8 +2209,10 @@ __global__ void __launch_bounds__(256) pid_kernel(const PidArgs a)
 // randomization, kFlagsRK4Fixed + s Runge-Kutta with the compile-time subset s; kN > 0 a
 // compile-time environment size, -1 a runtime size in blocks of at most kSmallBlock
 // threads, 0 any block size. The first variant that fits a launch is taken.
+// Randomized steps of uniform batches of up to 32 drones run randomized_step_kernel instead.
 #define MDG_STEP_VARIANTS(X) \
-    X(7, 4) X(7, 64) X(3, 1) X(8, -1) X(8, 0) X(9, -1) X(9, 0) X(10, -1) X(10, 0) X(11, 4) X(11, -1) X(11, 0) X(23, 4)
+    X(7, 4) X(7, 64) X(3, 1) X(8, -1) X(8, 0) X(9, -1) X(9, 0) X(10, -1) X(10, 0) X(11, -1) X(11, 0) X(23, 4)
+#define MDG_ROLLOUT_VARIANTS(X) X(11, 4) MDG_STEP_VARIANTS(X)
 
 template <bool kObs>
 static void* step_kernel_ptr(int flags, int N, int block)
@@ -2049,6 +2294,17 @@ cudaError_t launch_step(const StepArgs& a, int n_tiles, int block, bool with_obs
     // batch) and per-rotor ground heights run in runtime-flag variants of their own
     int flags, N;
     variant_of(a, uniform_flags, flags, N);
+    if (flags == kFlagsDR && N > 0 && N <= 32) {
+        StepArgs r = a;
+        r.envs_per_tile = kDrawDrones / N;
+        bool local = true;
+        for (int k = 0; k < r.envs_per_tile; ++k) local = local && (k * N >> 5) == ((k * N + N - 1) >> 5);
+        r.uniform_bits = (a.uniform_bits & kTileAnyDW) | (local ? kTileWarpLocal : 0);
+        const void* fn = N == 4 ? (with_obs ? (const void*)randomized_step_kernel<true, 4> : (const void*)randomized_step_kernel<false, 4>)
+                                : (with_obs ? (const void*)randomized_step_kernel<true, -1> : (const void*)randomized_step_kernel<false, -1>);
+        void* args[] = {&r};
+        return launch_overlapped(fn, (a.n_envs + r.envs_per_tile - 1) / r.envs_per_tile, kDrawDrones + 32, args, 0, s);
+    }
     void* fn = with_obs ? step_kernel_ptr<true>(flags, N, block) : step_kernel_ptr<false>(flags, N, block);
     if (!fn && flags >= kFlagsRK4Fixed) {  // no compile-time Runge-Kutta variant for this size or block
         flags = kFlagsRK4;
@@ -2068,7 +2324,7 @@ static void* rollout_kernel_ptr(int flags, int N, int block)
     if ((flags == F || (F == 8 && flags < 8)) &&                                                                    \
         (NN == 0 || (block <= kSmallBlock && (NN == -1 || N == NN))))                         \
         return (void*)rollout_kernel<F, NN>;
-    MDG_STEP_VARIANTS(MDG_PICK)
+    MDG_ROLLOUT_VARIANTS(MDG_PICK)
 #undef MDG_PICK
     return nullptr;
 }
@@ -2085,7 +2341,7 @@ static cudaError_t rollout_setup()
     if ((e = cudaFuncSetAttribute(rollout_kernel<F, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
                                   smem)) != cudaSuccess)                                                   \
         return e;
-    MDG_STEP_VARIANTS(MDG_ATTR)
+    MDG_ROLLOUT_VARIANTS(MDG_ATTR)
 #undef MDG_ATTR
     if (dev >= 0 && dev < 64) done[dev] = true;
     return cudaSuccess;

@@ -256,3 +256,43 @@ def test_obs_bias_needs_randomization(cuda):
     h = mdg.Handle(sw.drones_per_env, sw.flags)
     with pytest.raises(mdg.MdgError):
         h.set_obs_bias(torch.zeros((sw.n, 12), device=cuda))
+
+
+@pytest.mark.parametrize("drones,envs,depth", [(1, 70, 1), (2, 33, 2), (3, 43, 4), (4, 17, 3), (5, 13, 5), (31, 5, 3),
+                                               (32, 3, 3), (33, 3, 3)])
+def test_step_kernels_agree_with_the_rollout(cuda, drones, envs, depth):
+    """Three randomized control steps one by one (uniform batches of up to 32 drones: the kernel with
+    a drawing warp; 33: the general one) against the same steps as one rollout, whose drones draw
+    for themselves: partial blocks, environments across warps, histories of 1 to 5 rows, every
+    action type. The same float32 formulas in another order of noise and bias: heights are spread,
+    so 15 substeps amplify a rounding (6e-8) by far less than the 100 that 1e-5 allows; the rotor
+    speeds (to 2e4), histories and step counters alike."""
+    sw = spread_heights(wl.full_aero(201, n_envs=envs, drones=drones))
+    types = wl.all_action_types(202, envs)
+    table = wl.dr_table(203, envs, depth=depth)
+    K = 3
+    actions = torch.as_tensor(np.stack([wl.typed_actions(sw.drones_per_env, types, 204, k, HOVER, P.mass * P.g)
+                                        for k in range(K)]), device=cuda)
+    got = []
+    for rollout in (False, True):
+        h = mdg.Handle(sw.drones_per_env, sw.flags)
+        h.set_action_types(types)
+        live = h.new_randomization_state(depth, cuda)
+        h.set_randomization(torch.as_tensor(table, device=cuda), *live, seed=SEED)
+        bias = _bias(h, sw, cuda)
+        h.set_obs_bias(bias)
+        state = mdg.pack_state(sw.p, sw.q, sw.v, sw.w, device=cuda)
+        kin = torch.empty((K, sw.n, mdg.KIN_DIM), device=cuda)
+        idx = torch.empty((K, sw.n, mdg.NBR_K), dtype=torch.int32, device=cuda)
+        rel = torch.empty((K, sw.n, mdg.NBR_K * mdg.NBR_FEAT), device=cuda)
+        if rollout:
+            h.rollout(state, actions, mdg.ACT_MIXED, 5, K, mdg.OBS_EVERY_STEP, kin, idx, rel)
+        else:
+            for k in range(K):
+                h.step_obs(state, actions[k], mdg.ACT_MIXED, 5, kin[k], idx[k], rel[k])
+        assert h.status()[0] == mdg.OK
+        got.append((state, kin, rel, *live, idx))
+    a, b = got
+    assert torch.equal(a[4].isnan(), b[4].isnan()) and torch.equal(a[-1], b[-1])
+    for name, x, y in zip(("state", "kin", "rel", "motor", "history", "wind"), a, b):
+        np.testing.assert_allclose(x.cpu().numpy(), y.cpu().numpy(), rtol=1e-5, atol=1e-5, err_msg=name)

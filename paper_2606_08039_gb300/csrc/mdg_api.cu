@@ -256,6 +256,10 @@ int set_block(mdg_ctx* h, int block)
     }
     h->d_tiles = d_tiles;
     h->n_tiles = (int)tiles.size();
+    h->tile_pairs = true;
+    for (const mdg::Tile& t : tiles)
+        for (int k = t.z; k < t.z + (t.w & mdg::kTileEnvMask); ++k)
+            h->tile_pairs = h->tile_pairs && mdg::pair_sources(h->h_off[k] - t.x, h->h_off[k + 1] - h->h_off[k]);
     h->block = block;
     // Uniform batches (all environments of one size N > 0): the kernels compute the tiles
     // arithmetically (block / N environments per block), which the greedy packing matches.
@@ -341,6 +345,7 @@ int ensure_rollout_tables(mdg_ctx* h)
         bool dw = false;
         for (int32_t k = 0; k < h->n_envs; ++k) dw = dw || (h->h_flags[k] & MDG_DW);
         h->item_cost.assign(h->n_items, item_chain(h->uniform_N, dw ? MDG_DW : 0u));
+        h->item_pairs = h->tile_pairs;
     } else {
         const int cap = h->item_cap > 0 && h->item_cap < h->block ? h->item_cap : h->block;
         std::vector<int> envs;
@@ -352,6 +357,7 @@ int ensure_rollout_tables(mdg_ctx* h)
             if (h->h_flags[a] != h->h_flags[b]) return h->h_flags[a] < h->h_flags[b];
             return a < b;
         });
+        h->item_pairs = true;
         std::vector<int4> items;
         std::vector<int> slot_goff(envs.size()), slot_loff(envs.size());
         std::vector<double> cost;
@@ -371,6 +377,7 @@ int ensure_rollout_tables(mdg_ctx* h)
                     c += (double)n * n;
                 }
                 if ((drones >> 5) != ((drones + n - 1) >> 5)) local = false;
+                h->item_pairs = h->item_pairs && mdg::pair_sources(drones, n);
                 c += n;
                 chain = std::max(chain, item_chain(n, h->h_flags[envs[i]]));
                 drones += n;
@@ -483,6 +490,7 @@ mdg::StepArgs base_args(mdg_ctx* h, float* state)
     a.uniform_bits = h->uniform_bits;
     a.setpoints = h->d_sp;
     a.rand = h->dr ? h->d_rand : nullptr;
+    a.pairs = h->tile_pairs;
     a.c = h->dc;
     return a;
 }
@@ -1125,6 +1133,7 @@ static int rollout_args(mdg_handle h, float* state, const float* actions, int32_
     if ((rc = ensure_rollout_tables(h)) != MDG_OK) return rc;
     *r = mdg::RolloutArgs{};
     r->s = base_args(h, state);
+    r->s.pairs = h->item_pairs;
     r->s.action = reinterpret_cast<const float4*>(actions);
     r->s.kin = obs_mode != MDG_OBS_NONE ? kin : nullptr;
     r->s.nbr_idx = obs_mode != MDG_OBS_NONE ? reinterpret_cast<int4*>(nbr_idx) : nullptr;

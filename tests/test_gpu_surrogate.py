@@ -589,6 +589,37 @@ def test_surrogate_step_composes_its_parts(cuda, trained, recipe):
         assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(np.abs(want), 1.0)), np.abs(got - want).max()
 
 
+@pytest.mark.parametrize("sizes,block", [([1] * 33, None), ([3, 1, 5, 2, 33], None), ([64] * 3, None), ([7] * 11, 1024),
+                                         ([1000, 24], None)])
+def test_transition_rows_at_warp_edges(cuda, sizes, block):
+    """The staged rows of partial warps, uneven tiles and the largest block: the inputs are the
+    state's and the RPMs' own values, the change is the difference of the states, exactly, and
+    nothing beyond the rows is written."""
+    dpe = np.array(sizes, np.int32)
+    n = int(dpe.sum())
+    p, q, v, w = wl.random_states(501, n, pos_scale=3.0, z0=4.0)
+    h = mdg.Handle(dpe, np.full(len(dpe), 3, np.uint32))
+    if block:
+        h.set_block_size(block)
+    s0 = mdg.pack_state(p, q, v, w, device=cuda)
+    s1 = s0.clone()
+    rpm = torch.as_tensor(wl.rpm_actions(502, n, 0, 14468.0), device=cuda)
+    scale = torch.as_tensor(wl.uniform_range(0.9, 1.1, 503, 12, 0, np.arange(n, dtype=np.uint64)[:, None],
+                                             np.arange(4, dtype=np.uint64)[None, :]), device=cuda)
+    applied = torch.empty((n, 4), device=cuda)
+    buf = [torch.full((n * m + 64,), 7.0, device=cuda) for m in (mdg.MLP_IN, mdg.MLP_OUT)]
+    raw, delta = (b[:n * m].reshape(n, m) for b, m in zip(buf, (mdg.MLP_IN, mdg.MLP_OUT)))
+    h.transition(s1, rpm, applied, raw, delta, rpm_scale=scale)
+    assert torch.equal(applied, rpm * scale)
+    assert torch.equal(raw[:, :13], sg.state13(s0)) and torch.equal(raw[:, 13:17], applied)
+    assert torch.equal(delta, sg.state13(s1) - sg.state13(s0))
+    _, idx, rel = h.new_obs(cuda)
+    kin = torch.empty((n, mdg.KIN_DIM), device=cuda)
+    h.obs(s0, kin, idx, rel)
+    assert torch.equal(raw[:, 17:], rel)
+    assert all(torch.all(b[n * m:] == 7.0) for b, m in zip(buf, (mdg.MLP_IN, mdg.MLP_OUT)))
+
+
 @pytest.mark.parametrize("N", [130, 1024, 1025, 40003, 600001])
 def test_fit_normalization_at_tile_edges(cuda, N):
     """Row counts around the tiles' sizes and, at 600001, a sample stride of 2: statistics and rows

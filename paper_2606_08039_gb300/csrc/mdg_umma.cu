@@ -365,7 +365,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t bar0 = smem_u32(&bars[0]);
     auto bar = [bar0](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile int* abort = &s_abort;
-    const int n_pairs = (n_tiles + 1) / 2;
+    // This block's pairs of tiles (2k, 2k + 1), `whole` rounds of the grid; then, of the tiles that
+    // are left, one alone where the grid has a block for each of them, else one more pair. A lone
+    // tile takes two thirds of a pair's time (pairs in the last round, then lone tiles; 152 SMs):
+    // 16 tiles 17.5 us -> 14.2, 152 tiles 18.8 -> 14.7, 340 tiles 31.3 -> 26.9, 1024 tiles 56.2 ->
+    // 51.7, 1563 tiles 81.2 -> 76.2; more than half a round left (200, 512 tiles) as before. A lone
+    // tile is always a block's last: the barriers of a pair's second tile miss no phase.
+    const int grid = gridDim.x, whole = n_tiles / (2 * grid), left = n_tiles - 2 * grid * whole;
+    const bool lone = left <= grid;
+    const int n_steps = whole + ((int)blockIdx.x < (lone ? left : (left + 1) / 2) ? 1 : 0);
+    auto first_tile = [&](int s) {
+        return lone && s == whole ? 2 * grid * whole + (int)blockIdx.x : 2 * ((int)blockIdx.x + s * grid);
+    };
+    auto has_second = [&](int s) { return !(lone && s == whole) && first_tile(s) + 1 < n_tiles; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPNumBars; ++i) {
@@ -390,19 +402,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             int issued = 0, x_issued0 = 0, x_issued1 = 0;
             bool ok = true;
-            auto load_x = [&](int pr, int t) {
+            auto load_x = [&](int ta, int t) {
                 mbar_expect_tx(bar(kPBarXFull + t), kChunkBytes);
-                tma_rows(act0 + (uint32_t)t * 4 * kChunkBytes, &xmap, (2 * pr + t) * kRows, bar(kPBarXFull + t));
+                tma_rows(act0 + (uint32_t)t * 4 * kChunkBytes, &xmap, (ta + t) * kRows, bar(kPBarXFull + t));
                 if (t) ++x_issued1; else ++x_issued0;
             };
-            if (blockIdx.x < n_pairs) {  // the grid never exceeds the pair count
-                load_x(blockIdx.x, 0);
-                if (2 * blockIdx.x + 1 < n_tiles) load_x(blockIdx.x, 1);
+            if (n_steps > 0) {
+                load_x(first_tile(0), 0);
+                if (has_second(0)) load_x(first_tile(0), 1);
             }
-            int s = 0;  // pairs of this block
-            for (int pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x, ++s) {
-                const int next = pr + (int)gridDim.x;
-                const bool hasB = 2 * pr + 1 < n_tiles;
+            for (int s = 0; s < n_steps && ok; ++s) {  // pairs of this block
+                const int ta = first_tile(s);
+                const bool hasB = has_second(s);
                 for (int k = 0; k < kPLoadsPerPair; ++k) {
                     const int n = kPLoadsPerPair * s + k, slot = k % kPSlots;
                     if (n >= kPSlots)
@@ -418,13 +429,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                         // this pair's inputs go into their chunk 0
                         ok = mbar_spin(bar(kPBarActFree + 0), (s - 1) & 1, abort, status, 0, spin_limit);
                         if (!ok) break;
-                        load_x(pr, 0);
+                        load_x(ta, 0);
                         ok = mbar_spin(bar(kPBarActFree + 1), (s - 1) & 1, abort, status, 0, spin_limit);
                         if (!ok) break;
-                        if (hasB) load_x(pr, 1);
-                    } else if (k == 2 && next < n_pairs) {
-                        tma_rows_prefetch(&xmap, 2 * next * kRows);
-                        if (2 * next + 1 < n_tiles) tma_rows_prefetch(&xmap, (2 * next + 1) * kRows);
+                        if (hasB) load_x(ta, 1);
+                    } else if (k == 2 && s + 1 < n_steps) {
+                        tma_rows_prefetch(&xmap, first_tile(s + 1) * kRows);
+                        if (has_second(s + 1)) tma_rows_prefetch(&xmap, (first_tile(s + 1) + 1) * kRows);
                     }
                 }
             }
@@ -476,8 +487,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int k = 1; k < 4; ++k) mma_bf16_ss(d, ad + 2 * k, wd + 2 * k, id, 1);
             };
-            for (int pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x, ++s) {
-                const bool hasB = 2 * pr + 1 < n_tiles;
+            for (; s < n_steps && ok; ++s) {
+                const bool hasB = has_second(s);
                 const int nt = hasB ? 2 : 1;
                 // layer 1: the inputs in chunk 0 of each tile's activation buffer, one W1 chunk (load 0)
                 ok = wfull(0);
@@ -557,8 +568,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int sw = row & 7;
         uint32_t n_acc[2] = {0u, 0u};
         bool ok = true;
-        for (int pr = blockIdx.x; pr < n_pairs && ok; pr += gridDim.x) {
-            const bool hasB = 2 * pr + 1 < n_tiles;
+        for (int s = 0; s < n_steps && ok; ++s) {
+            const int ta = first_tile(s);
+            const bool hasB = has_second(s);
             const int nt = hasB ? 2 : 1;
             for (int l = 0; l < 3 && ok; ++l) {
                 const float* bias = master + w.b_off[l];
@@ -608,7 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
                 ++n_acc[t];
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const int tile = 2 * pr + t;
+                const int tile = ta + t;
                 if constexpr (!kApply) {
                     float v[8];
                     tmem_ld8(tmem + 256u * t + lane_off + p * 8, v);
@@ -722,8 +734,9 @@ cudaError_t mlp_forward_umma_pairs(const MlpView& w, const void* img, const void
     if ((e = input_map(&xmap, x, B)) != cudaSuccess) return e;
     int n_sm = 152;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    // one block per SM; fewer tiles: one each; fewer pairs but more tiles: one pair each
     const int n_pairs = (n_tiles + 1) / 2;
-    const int grid = n_pairs < n_sm ? n_pairs : n_sm;
+    const int grid = n_tiles <= n_sm ? n_tiles : n_pairs < n_sm ? n_pairs : n_sm;
     const MlpApply ap = apply ? *apply : MlpApply{};
     if (apply)
         mlp_umma_pair_kernel<true><<<grid, kThreads, kUmmaPairSmem, s>>>(

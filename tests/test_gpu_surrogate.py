@@ -180,6 +180,31 @@ def test_paired_kernel_equals_single_tile_kernel(cuda, n_tiles):
     assert np.all(np.abs(ys[1].cpu().numpy()[rows] - yo) <= bound)
 
 
+@pytest.mark.parametrize("n_tiles", [1, 2, 152, 153, 303, 304, 305, 340, 456, 457])
+def test_lone_last_tiles(cuda, n_tiles):
+    """The tiles left after the whole rounds of pairs, alone on a block each or in one more round of
+    pairs (152 SMs: the rule changes at 152 tiles left): a lone tile runs as the first of a pair, so
+    it equals the single-tile kernel's, as every even tile does; the others to the summation order's
+    bound of the test above."""
+    B, sms = 128 * n_tiles, torch.cuda.get_device_properties(0).multi_processor_count
+    m = mdg.MLP(B, _layers(4))
+    x = torch.as_tensor(_inputs(7, B), device=cuda).to(torch.bfloat16)
+    ys = []
+    for path in (mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_TCGEN05_PAIRS):
+        m.set_path(path)
+        y = torch.full((B, mdg.MLP_OUT_PAD), float("nan"), device=cuda)
+        m.forward(x, y)
+        assert m.status() == 0
+        ys.append(y.view(n_tiles, 128, mdg.MLP_OUT_PAD))
+    first = np.arange(n_tiles) % 2 == 0
+    whole = n_tiles // (2 * sms) * 2 * sms
+    if n_tiles - whole <= sms:
+        first[whole:] = True
+    first = torch.as_tensor(first, device=cuda)
+    assert torch.equal(ys[0][first], ys[1][first])
+    assert torch.all((ys[0] - ys[1]).abs() <= 1e-2 * torch.clamp(ys[0].abs(), min=1.0))
+
+
 @pytest.mark.parametrize("path,B", [(mdg.MLP_PATH_TCGEN05, 256), (mdg.MLP_PATH_TCGEN05, 1024),
                                     (mdg.MLP_PATH_MMA_SYNC, 256)])
 def test_gradients_and_loss_match_oracle(cuda, path, B):

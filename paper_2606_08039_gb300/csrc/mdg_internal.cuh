@@ -20,6 +20,17 @@ namespace mdg {
 #define MDG_CHECK(cond, status) true
 #endif
 
+#ifdef __CUDACC__
+// A step launched with programmatic stream serialisation may have its blocks placed while the grid
+// before it in the stream drains: it touches memory only after grid_wait (that grid has completed
+// and its writes are visible; at once when there is none). No kernel lets the next one in early:
+// its blocks then fill the SMs unevenly, and a step of one wave lasts as long as its fullest SM
+// (full aero, 8 steps in a graph: 55.9 us as plain launches, 54.6 so, 69.8 with a trigger at the
+// start, 59.2 with one before the stores).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+cudaError_t launch_overlapped(const void* fn, int grid, int block, void** args, size_t smem, cudaStream_t s);
+
 // Float32 copies of the model constants with the products the kernels need folded in
 // once on the host (in double precision, then rounded).
 struct DevConsts {
@@ -163,9 +174,11 @@ struct SurrogateArgs {
     const float* out_mean;       // [13]
     const float* out_std;        // [13]
     float ood_z;
-    unsigned* env_flag;          // [n_envs], zeroed before prepare
+    long long n_pad;             // rows of x
+    unsigned* env_flag;          // [n_envs], written by prepare
     int* fallback_list;          // [n_envs]
     int* fallback_count;         // [1], zeroed before prepare
+    int* n_fallback;             // fallback only: receives the count, or null
     float* raw;                  // features only: [n][41]
     const float4* rpm;           // features only: [n]
     const float4* rpm_scale;     // features only: [n], factors on rpm, or null

@@ -21,14 +21,6 @@ namespace {
 
 constexpr float kPi = 3.14159265358979323846f;
 
-// A step launched with programmatic stream serialisation may have its blocks placed while the grid
-// before it in the stream drains: it touches memory only after grid_wait (that grid has completed
-// and its writes are visible; at once when there is none). No kernel lets the next one in early:
-// its blocks then fill the SMs unevenly, and a step of one wave lasts as long as its fullest SM
-// (full aero, 8 steps in a graph: 55.9 us as plain launches, 54.6 so, 69.8 with a trigger at the
-// start, 59.2 with one before the stores).
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Approximate reciprocal and base-2 exponential of the special function unit
 // (rcp.approx.ftz.f32: relative error within 2^-23; ex2.approx.ftz.f32: within 2^-22).
 __device__ __forceinline__ float rcp_approx(float x)
@@ -2033,8 +2025,15 @@ __global__ void __launch_bounds__(1024) features_kernel(const SurrogateArgs sa)
 }
 
 // Before the network: action -> RPMs (PID state and plane 5 updated), standardised
-// inputs (bf16, zero padded to 64), and the out-of-distribution test of each drone; an
-// environment with any such drone is flagged once and listed for the fallback.
+// inputs (bf16, zero padded to 64; the rows up to the network's next tile of 128 zero), and the
+// out-of-distribution test of each drone: every environment's flag is written by its first drone,
+// which also lists it for the fallback. Bound by memory latency and the instructions of the
+// standardisation: a drone's 128-byte row leaves through shared memory with its warp's others as
+// one contiguous span, and an input's four constants are one 16-byte read. With the zeroed flags
+// and padding, the copied count and the launch gaps gone (50001 x 4 drones, the whole surrogate
+// step): 131.2 us -> 114.4.
+constexpr int kInputPitch = 9;                           // 16-byte words of a staged row: no bank conflict
+constexpr int kInputStage = 32 * kInputPitch * 16;       // bytes per warp
 __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const SurrogateArgs sa)
 {
     extern __shared__ float4 smem[];
@@ -2042,8 +2041,9 @@ __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const Surrogate
     const int B = blockDim.x;
     float4* s_pos = smem;
     float4* s_vel = smem + 2 * B;
-    int* s_off = reinterpret_cast<int*>(smem + 3 * B);
-    int* s_info = s_off + B + 1;
+    int* s_ood = reinterpret_cast<int*>(smem + 3 * B);  // by first drone of an environment
+    __shared__ float4 s_nrm[MDG_MLP_IN];                 // mean, 1/std, lo, hi of every input
+    grid_wait();
     const TileInfo tile = get_tile(a);
     const int t = threadIdx.x;
     const bool active = t < tile.n_drones;
@@ -2057,7 +2057,7 @@ __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const Surrogate
         if (a.act_type != MDG_ACT_RPM) s4 = a.state[4 * a.n + g];
         act = a.action[g];
     }
-    const EnvSlot env = tile_env(a, tile, s_off, s_info, t);
+    const EnvSlot env = tile_env(a, tile, nullptr, nullptr, t);  // one size: no tables
     Drone d;
     unpack_state(s0, s1, s2, s3, s4, d);
     float rpm[4] = {0.f, 0.f, 0.f, 0.f};
@@ -2084,23 +2084,18 @@ __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const Surrogate
     }
     s_pos[t] = make_float4(d.p[0], d.p[1], d.p[2], 0.f);
     s_vel[t] = make_float4(d.v[0], d.v[1], d.v[2], 0.f);
-    // the normalisation (mean, 1/std, lo, hi of every input), read by every drone
-    __shared__ float s_nrm[4][MDG_MLP_IN];
-    for (int i = t; i < 4 * MDG_MLP_IN; i += B) {
-        const int r = i / MDG_MLP_IN, k = i % MDG_MLP_IN;
-        const float* src = r == 0 ? sa.in_mean : r == 1 ? sa.in_inv_std : r == 2 ? sa.in_lo : sa.in_hi;
-        s_nrm[r][k] = src[k];
-    }
+    s_ood[t] = 0;
+    for (int i = t; i < MDG_MLP_IN; i += B) s_nrm[i] = make_float4(sa.in_mean[i], sa.in_inv_std[i], sa.in_lo[i], sa.in_hi[i]);
     __syncthreads();
-    bool ood = false;
+    uint4* stage = reinterpret_cast<uint4*>(reinterpret_cast<char*>(smem) + obs_stage_offset(B) + (t >> 5) * kInputStage);
+    const int lane = t & 31;
     if (active) {
+        bool ood = false;
         int bi[4];
         float f[24], x[41];
         knn_best4<0>(t - env.ls, d.p, s_pos + env.ls, env.N, bi);
         knn_features(bi, d, s_pos + env.ls, s_vel + env.ls, f);
         surrogate_inputs(d, rpm, f, x);
-        // the 128-byte input row in eight 16-byte stores of eight standardised inputs each
-        uint4* row = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(sa.x) + 64 * g);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             uint32_t o[4];
@@ -2109,23 +2104,33 @@ __global__ void __launch_bounds__(1024) surrogate_prepare_kernel(const Surrogate
                 const int k = 8 * q + 2 * i;
                 float z0 = 0.f, z1 = 0.f;
                 if (k < 41) {
-                    z0 = (x[k] - s_nrm[0][k]) * s_nrm[1][k];
-                    ood = ood || !(fabsf(z0) <= sa.ood_z) || !(x[k] >= s_nrm[2][k] && x[k] <= s_nrm[3][k]);
+                    const float4 c = s_nrm[k];
+                    z0 = (x[k] - c.x) * c.y;
+                    ood |= !(fabsf(z0) <= sa.ood_z) | !(x[k] >= c.z) | !(x[k] <= c.w);
                 }
                 if (k + 1 < 41) {
-                    z1 = (x[k + 1] - s_nrm[0][k + 1]) * s_nrm[1][k + 1];
-                    ood = ood || !(fabsf(z1) <= sa.ood_z) || !(x[k + 1] >= s_nrm[2][k + 1] && x[k + 1] <= s_nrm[3][k + 1]);
+                    const float4 c = s_nrm[k + 1];
+                    z1 = (x[k + 1] - c.x) * c.y;
+                    ood |= !(fabsf(z1) <= sa.ood_z) | !(x[k + 1] >= c.z) | !(x[k + 1] <= c.w);
                 }
                 const __nv_bfloat162 zz = __floats2bfloat162_rn(z0, z1);
                 o[i] = *reinterpret_cast<const uint32_t*>(&zz);
             }
-            row[q] = make_uint4(o[0], o[1], o[2], o[3]);
+            stage[kInputPitch * lane + q] = make_uint4(o[0], o[1], o[2], o[3]);
         }
-        if (ood) {
-            const int e = (int)((tile.first_drone + env.ls) / env.N);  // uniform batches
-            if (atomicOr(&sa.env_flag[e], 1u) == 0u) sa.fallback_list[atomicAdd(sa.fallback_count, 1)] = e;
-        }
+        if (ood) s_ood[env.ls] = 1;
     }
+    __syncthreads();
+    const int n16 = max(0, min(32, tile.n_drones - (t & ~31))) * 8;
+    uint4* x16 = static_cast<uint4*>(sa.x) + 8 * (g - lane);
+    for (int i = lane; i < n16; i += 32) x16[i] = stage[kInputPitch * (i >> 3) + (i & 7)];
+    if (active && t == env.ls) {
+        const unsigned flag = s_ood[t];
+        sa.env_flag[env.id] = flag;
+        if (flag) sa.fallback_list[atomicAdd(sa.fallback_count, 1)] = env.id;
+    }
+    if (blockIdx.x == gridDim.x - 1)  // the rows past the last drone
+        for (long long i = 8 * a.n + t; i < 8 * (long long)sa.n_pad; i += B) static_cast<uint4*>(sa.x)[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // After the network: state += de-standardised prediction (q renormalised) for every drone
@@ -2175,7 +2180,9 @@ __global__ void __launch_bounds__(128) surrogate_fallback_kernel(const Surrogate
     __shared__ float4 s_pos[4][2][32];
     const StepArgs& a = sa.s;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    grid_wait();
     const int count = *sa.fallback_count;
+    if (sa.n_fallback && blockIdx.x == 0 && threadIdx.x == 0) *sa.n_fallback = count;
     for (int item = blockIdx.x * 4 + wib; item < count; item += gridDim.x * 4) {
         const int e = sa.fallback_list[item];
         if (!MDG_CHECK(e >= 0 && e < a.n_envs, a.status)) continue;
@@ -2218,7 +2225,9 @@ __global__ void __launch_bounds__(1024) surrogate_fallback_block_kernel(const Su
     float4* s_pos = smem;  // [2][B]
     const StepArgs& a = sa.s;
     const int t = threadIdx.x, B = blockDim.x;
+    grid_wait();
     const int count = *sa.fallback_count;
+    if (sa.n_fallback && blockIdx.x == 0 && t == 0) *sa.n_fallback = count;
     for (int item = blockIdx.x; item < count; item += gridDim.x) {
         const int e = sa.fallback_list[item];
         if (!MDG_CHECK(e >= 0 && e < a.n_envs && a.uniform_N <= B, a.status)) continue;
@@ -2361,7 +2370,7 @@ static void variant_of(const StepArgs& a, int uniform_flags, int& flags, int& N)
 
 // A launch that may overlap the end of the kernel before it in the stream (grid_wait). Back to back
 // steps otherwise pay the launch latency and the placing of their blocks each time.
-static cudaError_t launch_overlapped(const void* fn, int grid, int block, void** args, size_t smem, cudaStream_t s)
+cudaError_t launch_overlapped(const void* fn, int grid, int block, void** args, size_t smem, cudaStream_t s)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2489,12 +2498,12 @@ cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cuda
 cudaError_t launch_surrogate_prepare(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s)
 {
     if (n_tiles == 0) return cudaSuccess;
-    const size_t smem = tile_smem_bytes(block);
+    const size_t smem = obs_stage_offset(block) + (size_t)(block / 32) * kInputStage;
     cudaError_t e =
         cudaFuncSetAttribute(surrogate_prepare_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    surrogate_prepare_kernel<<<n_tiles, block, smem, s>>>(a);
-    return cudaGetLastError();
+    void* args[] = {const_cast<SurrogateArgs*>(&a)};
+    return launch_overlapped((const void*)surrogate_prepare_kernel, n_tiles, block, args, smem, s);
 }
 
 cudaError_t launch_reset(const ResetArgs& r, cudaStream_t s)
@@ -2517,19 +2526,19 @@ cudaError_t launch_surrogate_fallback(const SurrogateArgs& a, cudaStream_t s)
 {
     if (a.s.n == 0) return cudaSuccess;
     const int N = a.s.uniform_N;
+    void* args[] = {const_cast<SurrogateArgs*>(&a)};
     if (N <= 32 && !a.s.c.rk4) {  // one warp per environment
         int blocks = (a.s.n_envs + 3) / 4;
         if (blocks > 152 * 8) blocks = 152 * 8;
-        surrogate_fallback_kernel<<<blocks, 128, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_overlapped((const void*)surrogate_fallback_kernel, blocks, 128, args, 0, s);
     }
     // one block per environment, grid-stride over the listed environments
     const int B = (N + 31) / 32 * 32;
     int blocks = a.s.n_envs < 152 * 4 ? a.s.n_envs : 152 * 4;
     const size_t smem = (size_t)2 * B * sizeof(float4);
-    if (a.s.c.rk4) surrogate_fallback_block_kernel<true><<<blocks, B, smem, s>>>(a);
-    else surrogate_fallback_block_kernel<false><<<blocks, B, smem, s>>>(a);
-    return cudaGetLastError();
+    const void* fn = a.s.c.rk4 ? (const void*)surrogate_fallback_block_kernel<true>
+                               : (const void*)surrogate_fallback_block_kernel<false>;
+    return launch_overlapped(fn, blocks, B, args, smem, s);
 }
 
 cudaError_t launch_obs(const StepArgs& a, int n_tiles, int block, cudaStream_t s)

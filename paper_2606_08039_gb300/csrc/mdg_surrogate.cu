@@ -127,6 +127,17 @@ cudaError_t forward_umma(mdg_mlp m, const void* x, int B, float* y, uint32_t* st
     return mdg::mlp_forward_umma(m->view(), m->img, x, B, y, status, m->wait_limit, m->spin_limit, s);
 }
 
+// A 4-byte aligned address in this device's own memory, which its kernels may write.
+bool on_device(const void* p, int device)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device && (reinterpret_cast<uintptr_t>(p) & 3u) == 0;
+}
+
 bool batch_ok(mdg_mlp m, int B) { return B > 0 && B % 128 == 0 && B <= m->max_batch; }
 
 struct Guard {
@@ -478,11 +489,10 @@ int mdg_surrogate_step(mdg_handle h, mdg_mlp m, float* state, const float* actio
     a.env_flag = m->env_flag;
     a.fallback_list = m->fb_list;
     a.fallback_count = m->fb_count;
-    cudaError_t e = cudaMemsetAsync(m->env_flag, 0, (size_t)h->n_envs * 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->fb_count, 0, 4, s);
-    if (e == cudaSuccess && n_pad > h->n_drones)  // padding rows of the network input
-        e = cudaMemsetAsync(m->x + (size_t)h->n_drones * MDG_MLP_IN_PAD, 0,
-                            (size_t)(n_pad - h->n_drones) * MDG_MLP_IN_PAD * 2, s);
+    a.n_pad = n_pad;
+    const bool direct = n_fallback && on_device(n_fallback, m->device);  // else copied below
+    a.n_fallback = direct ? n_fallback : nullptr;
+    cudaError_t e = cudaMemsetAsync(m->fb_count, 0, 4, s);
     bool fused = false;
     if (e == cudaSuccess) e = mdg::launch_surrogate_prepare(a, h->n_tiles, h->block, s);
     if (e == cudaSuccess) {
@@ -501,7 +511,7 @@ int mdg_surrogate_step(mdg_handle h, mdg_mlp m, float* state, const float* actio
     }
     if (e == cudaSuccess && !fused) e = mdg::launch_surrogate_apply(a, s);
     if (e == cudaSuccess) e = mdg::launch_surrogate_fallback(a, s);
-    if (e == cudaSuccess && n_fallback) e = cudaMemcpyAsync(n_fallback, m->fb_count, 4, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess && n_fallback && !direct) e = cudaMemcpyAsync(n_fallback, m->fb_count, 4, cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_surrogate_step");
 }
 

@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = s_tmem;
+    grid_wait();  // the inputs, the state and the weight image may come from the launch before
 
     if (warp == kProdWarp) {
         // ---------------- producer (one thread) ----------------
@@ -737,14 +738,13 @@ cudaError_t mlp_forward_umma_pairs(const MlpView& w, const void* img, const void
     // one block per SM; fewer tiles: one each; fewer pairs but more tiles: one pair each
     const int n_pairs = (n_tiles + 1) / 2;
     const int grid = n_tiles <= n_sm ? n_tiles : n_pairs < n_sm ? n_pairs : n_sm;
-    const MlpApply ap = apply ? *apply : MlpApply{};
-    if (apply)
-        mlp_umma_pair_kernel<true><<<grid, kThreads, kUmmaPairSmem, s>>>(
-            xmap, y, n_tiles, static_cast<const uint8_t*>(img), w.master, w, status, wait_limit, spin_limit, ap);
-    else
-        mlp_umma_pair_kernel<false><<<grid, kThreads, kUmmaPairSmem, s>>>(
-            xmap, y, n_tiles, static_cast<const uint8_t*>(img), w.master, w, status, wait_limit, spin_limit, ap);
-    return cudaGetLastError();
+    MlpApply ap = apply ? *apply : MlpApply{};
+    const uint8_t* image = static_cast<const uint8_t*>(img);
+    const float* master = w.master;
+    MlpView view = w;
+    void* args[] = {&xmap, &y, (void*)&n_tiles, &image, &master, &view, &status, &wait_limit, &spin_limit, &ap};
+    return launch_overlapped(apply ? (const void*)mlp_umma_pair_kernel<true> : (const void*)mlp_umma_pair_kernel<false>,
+                             grid, kThreads, args, kUmmaPairSmem, s);
 }
 
 cudaError_t mlp_forward_umma(const MlpView& w, const void* img, const void* x, int B, float* y, uint32_t* status,

@@ -705,3 +705,36 @@ def test_fit_normalization_without_usable_rows(cuda):
         with pytest.raises(mdg.MdgError):
             m.fit_normalization(raw, delta, x, t)
         assert torch.all(x == 1) and torch.all(t == 1)
+
+
+@pytest.mark.parametrize("size,envs,block", [(1, 300, None), (3, 43, None), (4, 33, 32), (7, 150, 1024), (33, 9, None),
+                                             (1000, 3, None)])
+def test_fallback_flags_at_tile_edges(cuda, size, envs, block):
+    """Environments over uneven tiles and blocks, every third with one drone (another place in each)
+    outside the box: exactly those take the integrator and are counted, also when the flags of an
+    earlier step are still in the workspace; the others change by the network's prediction, here
+    scaled to nothing, so their states stay as they were, exactly."""
+    n = size * envs
+    p, q, v, w = wl.random_states(511, n, pos_scale=3.0, z0=4.0)
+    bad = np.arange(envs) % 3 == 0
+    out = p.copy()
+    out[(np.arange(envs) * size + np.arange(envs) % size)[bad], 2] = 200.0
+    h = mdg.Handle(np.full(envs, size, np.int32), np.zeros(envs, np.uint32))
+    if block:
+        h.set_block_size(block)
+    m = mdg.MLP((n + 127) // 128 * 128, _layers(4))
+    lo, hi = np.full(mdg.MLP_IN, -1e30), np.full(mdg.MLP_IN, 1e30)
+    hi[2] = 100.0
+    m.set_normalization(np.zeros(mdg.MLP_IN), np.ones(mdg.MLP_IN), np.zeros(mdg.MLP_OUT), np.full(mdg.MLP_OUT, 1e-30), lo, hi)
+    rpm = torch.zeros((n, 4), device=cuda)  # free fall
+    nfb = torch.full((1,), -1, dtype=torch.int32, device=cuda)
+    for pos, flagged in ((out, bad), (p, np.zeros(envs, bool)), (out, bad)):
+        s0 = mdg.pack_state(pos, q, v, w, device=cuda)
+        s1 = s0.clone()
+        m.step(h, s1, rpm, mdg.ACT_RPM, 5, 1e30, nfb)
+        assert int(nfb) == flagged.sum()
+        a, b = (sg.state13(s).view(envs, size, 13)[:, :, [0, 1, 2, 7, 8, 9, 10, 11, 12]] for s in (s0, s1))
+        same = (a == b).all(dim=2)
+        f = torch.as_tensor(flagged, device=cuda)
+        assert torch.all(same[~f]) and not torch.any(same[f])
+    assert m.status() == 0 and h.status()[0] == mdg.OK

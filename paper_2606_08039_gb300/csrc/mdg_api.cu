@@ -118,6 +118,7 @@ DevConsts make_dev_consts(const mdg_constants& c)
     for (int i = 0; i < 3; ++i) {
         d.J[i] = (float)J[i];
         d.inv_J[i] = (float)(1.0 / J[i]);
+        d.gyro[i] = (float)((J[(i + 2) % 3] - J[(i + 1) % 3]) / J[i]);
     }
     d.gnd_k = (float)(c.c_gnd * (c.prop_radius / 4.0) * (c.prop_radius / 4.0));
     d.h_clip = (float)c.h_clip;
@@ -141,6 +142,7 @@ DevConsts make_dev_consts(const mdg_constants& c)
     d.pos_iclamp = (float)c.pos_iclamp;
     d.att_iclamp = (float)c.att_iclamp;
     d.dt_sim = (float)c.dt_sim;
+    d.dt_mass = (float)(c.dt_sim / c.mass);
     d.dt_ctrl = (float)c.dt_ctrl;
     const double maxrpm = sqrt(c.thrust2weight * c.mass * c.g / (4.0 * c.kf));
     d.max_rpm = (float)maxrpm;

@@ -37,6 +37,7 @@ struct DevConsts {
     float mass, inv_mass, g, inv_g;
     float kf, km, l_sqrt2;            // Eq. motor: k_f, k_m, L/sqrt(2)
     float J[3], inv_J[3];
+    float gyro[3];                    // (J_z - J_y) / J_x, (J_x - J_z) / J_y, (J_y - J_x) / J_z
     float gnd_k;                      // Eq. ground: C_gnd (r_p/4)^2
     float h_clip;
     float drag_k;                     // Eq. drag: 2 pi / 60 (RPM -> rad/s)
@@ -46,6 +47,7 @@ struct DevConsts {
     float pos_kp[3], pos_ki[3], pos_kd[3], pos_iclamp;
     float att_kp[3], att_ki[3], att_kd[3], att_iclamp;
     float dt_sim, dt_ctrl;
+    float dt_mass;                    // dt_sim / mass
     float max_rpm, f_max, inv_kf;     // PID output clip: f_i in [0, k_f MAX_RPM^2]
     float hover_rpm;                  // normalized actions: 0 -> HOVER_RPM
     float alloc_xy, alloc_z;          // inverse mixing: sqrt(2)/L (X) or 2/L (+), and k_f/k_m

@@ -142,7 +142,6 @@ DevConsts make_dev_consts(const mdg_constants& c)
     d.pos_iclamp = (float)c.pos_iclamp;
     d.att_iclamp = (float)c.att_iclamp;
     d.dt_sim = (float)c.dt_sim;
-    d.dt_mass = (float)(c.dt_sim / c.mass);
     d.dt_ctrl = (float)c.dt_ctrl;
     const double maxrpm = sqrt(c.thrust2weight * c.mass * c.g / (4.0 * c.kf));
     d.max_rpm = (float)maxrpm;

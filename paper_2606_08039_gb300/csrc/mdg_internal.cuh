@@ -47,7 +47,6 @@ struct DevConsts {
     float pos_kp[3], pos_ki[3], pos_kd[3], pos_iclamp;
     float att_kp[3], att_ki[3], att_kd[3], att_iclamp;
     float dt_sim, dt_ctrl;
-    float dt_mass;                    // dt_sim / mass
     float max_rpm, f_max, inv_kf;     // PID output clip: f_i in [0, k_f MAX_RPM^2]
     float hover_rpm;                  // normalized actions: 0 -> HOVER_RPM
     float alloc_xy, alloc_z;          // inverse mixing: sqrt(2)/L (X) or 2/L (+), and k_f/k_m

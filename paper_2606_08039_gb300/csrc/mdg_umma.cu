@@ -634,18 +634,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                     out[1] = make_float4(v[4] + b4[4], v[5] + b4[5], v[6] + b4[6], v[7] + b4[7]);
                     continue;
                 } else {
-                // the state update instead of y: the warps of column part 0 read the row's first
-                // 16 columns (the 13 outputs) and update their drone; the others only release
+                // the state update instead of y: four warps (column part 0 for tile A, part 1 for B, so
+                // that one tile's update does not wait for the other's; a surrogate step of 50001 x 4
+                // 112.9 us -> 111.4, of 16384 x 4 48.0 -> 46.8) read the row's first 16 columns (the
+                // 13 outputs) and update their drone; the others only release. Loading the state
+                // ahead of the wait spills registers (+3 us), fetching it to L1 gave nothing.
                 float v[16];
-                if (p == 0) {
+                if (p == t) {
                     tmem_ld8(tmem + 256u * t + lane_off, v);
                     tmem_ld8(tmem + 256u * t + lane_off + 8, v + 8);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kPBarAccDrained + t));
-                const long long g = (long long)tile * kRows + row;
-                if (p == 0 && g < ap.n && !ap.env_flag[g / ap.uniform_N]) {
+                const int g = tile * kRows + row;  // rows are an int
+                if (p == t && g < ap.n && !ap.env_flag[g / ap.uniform_N]) {
                     const float* b = master + w.b_off[3];
                     float dl[13];
 #pragma unroll

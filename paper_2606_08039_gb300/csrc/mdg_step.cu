@@ -2348,7 +2348,12 @@ static void* step_kernel_ptr(int flags, int N, int block, bool pairs)
     return nullptr;
 }
 
-// Opt the tile kernels in to the shared memory of the largest block, once per device.
+static size_t features_smem_bytes(int B) { return obs_stage_offset(B) + (size_t)(B / 32) * kRawStage; }
+static size_t prepare_smem_bytes(int B) { return obs_stage_offset(B) + (size_t)(B / 32) * kInputStage; }
+
+// Opt the tile kernels in to the shared memory of the largest block, once per device: the limit
+// belongs to the kernel and not to a launch, so that a launch that set it to its own size could
+// lower it under a larger one that another host thread is about to make.
 static cudaError_t tile_kernels_setup()
 {
     static bool done[64] = {};
@@ -2365,7 +2370,11 @@ static cudaError_t tile_kernels_setup()
         return e;
     MDG_STEP_VARIANTS(MDG_ATTR)
 #undef MDG_ATTR
-    if ((e = cudaFuncSetAttribute(obs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(obs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)features_smem_bytes(1024))) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(surrogate_prepare_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)prepare_smem_bytes(1024))) != cudaSuccess)
         return e;
     if (dev >= 0 && dev < 64) done[dev] = true;
     return cudaSuccess;
@@ -2509,22 +2518,19 @@ cudaError_t launch_rollout(const RolloutArgs& r, int block, int uniform_flags, i
 cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s)
 {
     if (n_tiles == 0) return cudaSuccess;
-    const size_t smem = obs_stage_offset(block) + (size_t)(block / 32) * kRawStage;
-    cudaError_t e = cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = tile_kernels_setup();
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<SurrogateArgs*>(&a)};
-    return launch_overlapped((const void*)features_kernel, n_tiles, block, args, smem, s);
+    return launch_overlapped((const void*)features_kernel, n_tiles, block, args, features_smem_bytes(block), s);
 }
 
 cudaError_t launch_surrogate_prepare(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s)
 {
     if (n_tiles == 0) return cudaSuccess;
-    const size_t smem = obs_stage_offset(block) + (size_t)(block / 32) * kInputStage;
-    cudaError_t e =
-        cudaFuncSetAttribute(surrogate_prepare_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = tile_kernels_setup();
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<SurrogateArgs*>(&a)};
-    return launch_overlapped((const void*)surrogate_prepare_kernel, n_tiles, block, args, smem, s);
+    return launch_overlapped((const void*)surrogate_prepare_kernel, n_tiles, block, args, prepare_smem_bytes(block), s);
 }
 
 cudaError_t launch_reset(const ResetArgs& r, cudaStream_t s)

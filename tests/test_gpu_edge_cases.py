@@ -2,6 +2,8 @@
 non-finite state reporting and argument errors, each checked against the oracle where a
 result exists."""
 import math
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -278,3 +280,47 @@ def test_results_do_not_depend_on_the_tile_size(cuda):
     # the variants sum the downwash in different orders: within the per-substep tolerances
     # over the 15 substeps of the three control steps
     assert_state_close(oracle_arrays(a[0])[0], oracle_arrays(b[0])[0], scale=15, what="variants")
+
+
+@pytest.mark.parametrize("call", ["features", "surrogate", "render"])
+def test_host_threads_with_handles_of_different_sizes(cuda, call):
+    """Two host threads, each with its own handle, stream and buffers, whose launches need different
+    amounts of shared memory: neither's launch is refused for what the other one asked for."""
+    def worker(dpe, block, errors):
+        try:
+            torch.cuda.set_device(cuda)
+            h = mdg.Handle(dpe, np.zeros(len(dpe), np.uint32))
+            if block:
+                h.set_block_size(block)
+            p, q, v, w = wl.random_states(601, h.n, pos_scale=3.0, z0=4.0)
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                state = mdg.pack_state(p, q, v, w, device=cuda)
+                rpm = torch.full((h.n, 4), HOVER, device=cuda)
+                raw = torch.empty((h.n, mdg.MLP_IN), device=cuda)
+                frames = h.new_frames(cuda) if call == "render" else None
+                m = mdg.MLP((h.n + 127) // 128 * 128) if call == "surrogate" else None
+                if m:
+                    one_in, one_out = np.ones(mdg.MLP_IN), np.ones(mdg.MLP_OUT)
+                    m.set_normalization(0 * one_in, one_in, 0 * one_out, one_out, -1e30 * one_in, 1e30 * one_in)
+                start.wait(timeout=60)
+                end = time.monotonic() + 1.5
+                while time.monotonic() < end and not errors:
+                    if call == "features":
+                        h.features(state, rpm, raw)
+                    elif call == "surrogate":
+                        m.step(h, state, rpm, mdg.ACT_RPM, 1, 1e30)
+                    else:
+                        h.render(state, *frames)
+                stream.synchronize()
+        except Exception as e:  # reported by the test, not by the thread
+            errors.append(e)
+
+    sizes = [([1000], None), ([450], None)] if call == "render" else [([4] * 300, 1024), ([4] * 300, 32)]
+    errors, start = [], threading.Barrier(2)
+    threads = [threading.Thread(target=worker, args=(np.array(d, np.int32), b, errors)) for d, b in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors

@@ -356,9 +356,12 @@ int mdg_mlp_grad(mdg_mlp m, const uint16_t* x, const float* t, int32_t B, float*
         }
         tb.dy = m->dy;
         tb.loss = m->loss_part;
+        const bool direct = loss_out && on_device(loss_out, m->device);  // else copied below
         e = refresh_image(m, s);
         if (e == cudaSuccess)
-            e = mdg::mlp_grad_umma(m->view(), m->img, tb, x, B, t, m->loss, loss_out, m->grad, m->status, s);
+            e = mdg::mlp_grad_umma(m->view(), m->img, tb, x, B, t, m->loss, direct ? loss_out : nullptr, m->grad,
+                                   m->status, s);
+        if (direct) loss_out = nullptr;
     } else {
         float* zs[3] = {m->z[0], m->z[1], m->z[2]};
         void* hs[3] = {m->h[0], m->h[1], m->h[2]};
@@ -366,8 +369,8 @@ int mdg_mlp_grad(mdg_mlp m, const uint16_t* x, const float* t, int32_t B, float*
         e = cudaMemsetAsync(m->loss, 0, 4, s);
         if (e == cudaSuccess) e = mdg::mlp_forward(m->view(), x, B, zs, hs, m->y, t, m->dy, m->loss, s);
         if (e == cudaSuccess) e = mdg::mlp_backward(m->view(), x, B, zs, hs, m->dy, dzs, m->grad, s);
-        if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToDevice, s);
     }
+    if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_grad");
 }
 

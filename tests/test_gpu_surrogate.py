@@ -247,6 +247,26 @@ def test_gradients_over_uneven_tile_shares(cuda, B):
     test_gradients_and_loss_match_oracle(cuda, mdg.MLP_PATH_TCGEN05, B)
 
 
+@pytest.mark.parametrize("path", [mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_MMA_SYNC])
+def test_loss_at_any_address(cuda, path):
+    """The loss goes to any address that a copy can reach: one that is not 4-byte aligned (no kernel
+    stores to it) receives the same four bytes, and its neighbours stay as they were."""
+    B = 128
+    m = mdg.MLP(B, _layers(31))
+    m.set_train_path(path)
+    x = torch.as_tensor(_inputs(32, B), device=cuda).to(torch.bfloat16)
+    t = torch.full((B, mdg.MLP_OUT_PAD), 0.25, device=cuda)
+    loss = torch.zeros(1, device=cuda)
+    m.grad(x, t, loss)
+    buf = torch.full((12,), 7, dtype=torch.uint8, device=cuda)
+    stream = torch.cuda.current_stream().cuda_stream
+    assert mdg.lib().mdg_mlp_grad(m._m, x.data_ptr(), t.data_ptr(), B, buf.data_ptr() + 5, stream) == mdg.OK
+    got = buf.cpu().numpy()
+    # mma.sync adds its partial losses up with atomics, in any order
+    np.testing.assert_allclose(got[5:9].view(np.float32), loss.cpu().numpy(), rtol=0 if path == mdg.MLP_PATH_TCGEN05 else 1e-6)
+    assert float(loss) > 0 and np.all(np.delete(got, slice(5, 9)) == 7)
+
+
 def test_adam_refreshes_the_weight_image(cuda):
     """The forward pass after an Adam step equals, bit for bit, that of a network created with
     the updated parameters (whose image is built from their bf16 copies)."""

@@ -71,7 +71,6 @@ struct mdg_mlp_s {
     uint32_t* status = nullptr;
     int path = MDG_MLP_PATH_TCGEN05_PAIRS;
     uint8_t* img = nullptr;      // weight image of the tcgen05 kernel
-    bool img_stale = true;       // the bf16 weights changed since the image was built
     int wait_limit = MDG_MLP_DEFAULT_TRY_WAITS;  // bounded waits of the tcgen05 kernel
     int spin_limit = MDG_MLP_DEFAULT_POLLS;
     int train_path = MDG_MLP_PATH_TCGEN05;
@@ -107,21 +106,18 @@ void destroy_mlp(mdg_mlp m)
     delete m;
 }
 
-// The tcgen05 kernels read the weights from their image; rebuild it after mdg_mlp_set_params (Adam
-// refreshes it itself).
-cudaError_t refresh_image(mdg_mlp m, cudaStream_t s)
+// The bf16 copies and the weight image of the tcgen05 kernels, from the master parameters. The image
+// is rewritten by whatever writes the weights (here and by Adam, in its own kernel), so that it is
+// right in stream order, also when the calls around it were captured and not run, or failed.
+cudaError_t refresh_weights(mdg_mlp m, cudaStream_t s)
 {
-    if (!m->img_stale) return cudaSuccess;
-    const cudaError_t e = mdg::mlp_build_image(m->view(), m->img, s);
-    if (e == cudaSuccess) m->img_stale = false;
-    return e;
+    const cudaError_t e = mdg::mlp_refresh_bf16(m->view(), s);
+    return e == cudaSuccess ? mdg::mlp_build_image(m->view(), m->img, s) : e;
 }
 
 cudaError_t forward_umma(mdg_mlp m, const void* x, int B, float* y, uint32_t* status, cudaStream_t s,
                          const mdg::MlpApply* apply = nullptr)
 {
-    const cudaError_t e = refresh_image(m, s);
-    if (e != cudaSuccess) return e;
     if (m->path == MDG_MLP_PATH_TCGEN05_PAIRS)
         return mdg::mlp_forward_umma_pairs(m->view(), m->img, x, B, y, status, m->wait_limit, m->spin_limit, s, apply);
     return mdg::mlp_forward_umma(m->view(), m->img, x, B, y, status, m->wait_limit, m->spin_limit, s);
@@ -217,7 +213,7 @@ int mdg_mlp_create(int32_t max_batch, const float* init, mdg_mlp* out)
     alloc((void**)&m->img, mdg::mlp_image_bytes());
     alloc((void**)&m->loss_part, B / 16 * 4);
     if (e == cudaSuccess && init) e = cudaMemcpy(m->master, init, P * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = mdg::mlp_refresh_bf16(m->view(), 0);
+    if (e == cudaSuccess) e = refresh_weights(m, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         destroy_mlp(m);
@@ -249,8 +245,7 @@ int mdg_mlp_set_params(mdg_mlp m, const float* host_in)
     if (!m || !host_in) return fail(MDG_ERR_ARG, "mdg_mlp_set_params: NULL argument");
     Guard g(m->device);
     cudaError_t e = cudaMemcpy(m->master, host_in, (size_t)MDG_MLP_PARAMS * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = mdg::mlp_refresh_bf16(m->view(), 0);
-    m->img_stale = true;
+    if (e == cudaSuccess) e = refresh_weights(m, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_set_params");
 }
@@ -357,10 +352,7 @@ int mdg_mlp_grad(mdg_mlp m, const uint16_t* x, const float* t, int32_t B, float*
         tb.dy = m->dy;
         tb.loss = m->loss_part;
         const bool direct = loss_out && on_device(loss_out, m->device);  // else copied below
-        e = refresh_image(m, s);
-        if (e == cudaSuccess)
-            e = mdg::mlp_grad_umma(m->view(), m->img, tb, x, B, t, m->loss, direct ? loss_out : nullptr, m->grad,
-                                   m->status, s);
+        e = mdg::mlp_grad_umma(m->view(), m->img, tb, x, B, t, m->loss, direct ? loss_out : nullptr, m->grad, m->status, s);
         if (direct) loss_out = nullptr;
     } else {
         float* zs[3] = {m->z[0], m->z[1], m->z[2]};
@@ -380,7 +372,6 @@ int mdg_mlp_adam(mdg_mlp m, float lr, void* stream)
     if (!(lr > 0.f)) return fail(MDG_ERR_ARG, "mdg_mlp_adam: lr must be > 0");
     Guard g(m->device);
     m->step += 1;
-    m->img_stale = false;  // Adam writes every weight's place in the image
     cudaError_t e = mdg::mlp_adam(m->view(), m->img, m->grad, m->m, m->v, lr, m->step, (cudaStream_t)stream);
     return e == cudaSuccess ? MDG_OK : cuda_fail(e, "mdg_mlp_adam");
 }

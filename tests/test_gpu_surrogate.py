@@ -288,6 +288,39 @@ def test_adam_refreshes_the_weight_image(cuda):
         assert torch.equal(*ys)
 
 
+@pytest.mark.parametrize("path", [mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_TCGEN05_PAIRS])
+def test_weights_around_captured_calls(cuda, path):
+    """Calls that were captured and have not run change nothing: the forward pass after a captured,
+    unplayed training step equals that of another network with the same parameters, bit for bit. And
+    a captured forward pass reads the parameters set after its capture."""
+    B = 256
+    x = torch.as_tensor(_inputs(42, B), device=cuda).to(torch.bfloat16)
+    t = torch.full((B, mdg.MLP_OUT_PAD), 0.25, device=cuda)
+
+    def forward(net):
+        y = torch.empty((B, mdg.MLP_OUT_PAD), device=cuda)
+        net.forward(x, y)
+        return y
+    nets = [mdg.MLP(B, _layers(41)), mdg.MLP(B, _layers(41)), mdg.MLP(B, _layers(43))]
+    for net in nets:
+        net.set_path(path)
+    want = [forward(net) for net in nets[1:]]
+    m = nets[0]
+    train, infer = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(train):
+        m.grad(x, t)
+        m.adam(1e-2)
+    assert torch.equal(forward(m), want[0])
+    y = torch.zeros((B, mdg.MLP_OUT_PAD), device=cuda)
+    with torch.cuda.graph(infer):
+        m.forward(x, y)
+    m.set_params(nets[2].params())
+    infer.replay()
+    assert torch.equal(y, want[1])
+    train.replay()
+    assert not torch.equal(forward(m), want[1])
+
+
 def test_adam_matches_oracle(cuda):
     B = 128
     layers = _layers(6)

@@ -26,8 +26,18 @@ namespace mdg {
 // and its writes are visible; at once when there is none). No kernel lets the next one in early:
 // its blocks then fill the SMs unevenly, and a step of one wave lasts as long as its fullest SM
 // (full aero, 8 steps in a graph: 55.9 us as plain launches, 54.6 so, 69.8 with a trigger at the
-// start, 59.2 with one before the stores).
+// start, 59.2 with one before the stores). Such a kernel reads global memory with plain loads through
+// plain pointers, or through after_wait: a read-only load (__ldg, or one inferred from __restrict__)
+// counts as independent of every store, so that the compiler may move it above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The pointer as the result of a statement that follows the wait, so that nothing read through it, by
+// read-only loads either, can move above. For data that the kernel itself leaves alone.
+template <class T>
+__device__ __forceinline__ const T* after_wait(const T* p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 #endif
 cudaError_t launch_overlapped(const void* fn, int grid, int block, void** args, size_t smem, cudaStream_t s);
 

@@ -1116,7 +1116,7 @@ __device__ __forceinline__ void load_row(const float* dr, int env, float r[MDG_D
     const float4* p = reinterpret_cast<const float4*>(dr + (long long)env * MDG_DR_PARAMS);
 #pragma unroll
     for (int i = 0; i < MDG_DR_PARAMS / 4; ++i) {
-        const float4 v = __ldg(p + i);
+        const float4 v = p[i];
         r[4 * i] = v.x, r[4 * i + 1] = v.y, r[4 * i + 2] = v.z, r[4 * i + 3] = v.w;
     }
 }

@@ -150,3 +150,31 @@ def test_noalloc_source_names_no_device_allocation():
                         r"cudaHostAlloc|cudaMallocHost)\b", code)
     assert banned == []
     assert "cudaGetSymbolAddress" in code and "cudaStreamIsCapturing" in code
+
+
+def _code(name):
+    """A source file of the library without its comments."""
+    src = open(os.path.join(ROOT, "paper_2606_08039_gb300", "csrc", name)).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", src, flags=re.S))
+
+
+@pytest.mark.parametrize("name", ["mdg_step.cu", "mdg_train.cu", "mdg_umma.cu"])
+def test_kernels_that_wait_for_the_launch_before_use_plain_loads(name):
+    """A kernel that may start before the launch ahead of it has ended (grid_wait) reads what that one
+    writes: no read-only loads, which the compiler may move above the wait, by __restrict__ or by name, but
+    through a pointer that comes out of the wait (after_wait)."""
+    code = _code(name)
+    loads = re.findall(r"__ldg\(.*|ld\.global\.nc.*", code)
+    if name == "mdg_umma.cu":  # the paired kernel's hidden biases
+        assert "waited = after_wait(master);" in code and "float* bias = waited + w.b_off[l];" in code
+        assert loads == ["__ldg(reinterpret_cast<const float4*>(bias + col) + i);"]
+    else:
+        assert loads == []
+    waiting = 0
+    for kernel in re.split(r"\b__global__\b", code)[1:]:
+        body = kernel[kernel.index("{"):]
+        end = re.search(r"\n}", body).start()
+        if "grid_wait()" in body[:end]:
+            waiting += 1
+            assert "__restrict__" not in kernel[:kernel.index("{")], kernel[:200]
+    assert waiting >= 1

@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw,
                                                   uint32_t* __restrict__ keep, double* __restrict__ partial,
                                                   long long* __restrict__ box_rows)
 {
-    extern __shared__ float s_tile[];  // [2][kSubFloats]
+    extern __shared__ __align__(16) float s_tile[];  // [2][kSubFloats], filled 16 bytes at a time
     __shared__ float2 s_box[kCols];
     __shared__ uint32_t s_part[2][4], s_words[4];
     __shared__ double s_sum[4][kCols][2];
@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(256) zbox_kernel(const float* __restrict__ raw
                                                    long long N, const uint32_t* __restrict__ box, Stats* __restrict__ st,
                                                    uint32_t* __restrict__ keep, int* __restrict__ counts)
 {
-    extern __shared__ float s_tile[];
+    extern __shared__ __align__(16) float s_tile[];
     __shared__ float2 s_lim[kCols];
     __shared__ uint32_t s_part[2][4], s_words[4];
     for (int c = threadIdx.x; c < kCols; c += 256) s_lim[c] = make_float2(st->mean[c], st->limit[c]);
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const float* __restrict__ raw
                                                    const int* __restrict__ offsets, const Stats* __restrict__ st,
                                                    uint4* __restrict__ x, float4* __restrict__ t_out)
 {
-    extern __shared__ float s_tile[];
+    extern __shared__ __align__(16) float s_tile[];
     __shared__ uint8_t s_row[kSub];
     const int piece = threadIdx.x & 7, first = (threadIdx.x >> 3) & 15;
     const bool input = threadIdx.x < 128;

@@ -178,3 +178,16 @@ def test_kernels_that_wait_for_the_launch_before_use_plain_loads(name):
             waiting += 1
             assert "__restrict__" not in kernel[:kernel.index("{")], kernel[:200]
     assert waiting >= 1
+
+
+def test_dynamic_shared_memory_is_declared_aligned():
+    """Every kernel's dynamic shared memory, read or written 16 bytes at a time, asks for that alignment
+    by its type or by name: what lies before it (the kernel's static arrays) promises nothing."""
+    found = 0
+    for name in sorted(os.listdir(os.path.join(ROOT, "paper_2606_08039_gb300", "csrc"))):
+        if name.endswith((".cu", ".cuh")):
+            for decl in re.findall(r"extern __shared__ ([^;]*);", _code(name)):
+                align = re.match(r"__align__\((\d+)\)", decl)
+                assert decl.startswith("float4 ") or (align and int(align.group(1)) >= 16), f"{name}: {decl}"
+                found += 1
+    assert found >= 10

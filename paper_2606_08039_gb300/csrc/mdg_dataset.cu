@@ -93,17 +93,20 @@ __host__ __device__ inline float key_float(uint32_t k)
 #endif
 }
 
-// The standardisation of a transition set reads the set four times, each time as contiguous tiles
+// The standardisation of a transition set reads the set five times, each time as contiguous tiles
 // of rows copied into shared memory (or, for the finite test, straight through registers), and
-// keeps its decisions as one bit a row: finite; inside the trim box (with the moments of the
-// rows that are); inside the z limits (with their range); the training set written out. Bytes of
-// the four reads bound it: 216 B a row each, and 256 B a row written. Every number that a later
-// kernel needs stays on the device, so the host waits once, at the end. 2,000,003 rows: 7.1 ms
-// with a thread per row or per element (32 counting passes for the quantiles, FP64 shared-memory
-// atomics for the moments, 15 allocations and 8 waits), 1.0 ms now: finite 74 us (5.8 TB/s),
-// sample 58, selection 97, box and moments 179 (its arithmetic), z limits 79 (5.5 TB/s), training
-// set 142 (5.8 TB/s, both ways), the two scans and the statistics 30; the rest is the one
-// allocation and its release (150 us) and the host's copies.
+// keeps its decisions as one bit a row: finite; inside the trim box (with the sums of the rows
+// that are); those rows' squared deviations from the means; inside the z limits (with their range);
+// the training set written out. Bytes of the reads bound it, but for the sums: 216 B a row each,
+// and 256 B a row written. Every number that a later kernel needs stays on the device, so the host
+// waits once, at the end. 2,000,003 rows: 7.1 ms with a thread per row or per element (32 counting
+// passes for the quantiles, FP64 shared-memory atomics for the moments, 15 allocations and 8
+// waits), 1.1 ms now: finite 74 us (5.8 TB/s), sample 58, selection 97, box and sums 144, deviations
+// 157 (both their arithmetic), z limits 76 (5.7 TB/s), training set 141 (5.9 TB/s, both ways), the
+// two scans, means and statistics 35; the rest is the one allocation and its release (150 us) and
+// the host's copies. (One pass for sum and square about the middle of the box took 179 us instead of
+// the 301 of two, but lost deviations to cancellation and overflow where the box is wide: without a
+// limit, margin = inf, one of 0.05 about 1e4 came out 8e-5 of itself off and a column of size 1e25 as constant.)
 
 // Counts of the set: finite rows, rows inside the trim box, rows kept.
 struct Counts {
@@ -112,6 +115,9 @@ struct Counts {
 
 struct Stats {
     float box_lo[kCols], box_hi[kCols];  // the trim box of every column
+    uint32_t box_min[kCols], box_max[kCols];  // range of the rows inside it, as float keys
+    double mean64[kCols];
+    float pivot[kCols], scale[kCols];  // the deviations' frame
     float mean[kCols], inv_std[kCols], std_[kCols];
     float limit[kCols];  // the largest |v - mean| that passes: |v - mean| / std <= the column's z limit
     uint32_t key_min[kIn], key_max[kIn];  // range of the kept rows, as float keys
@@ -287,6 +293,7 @@ __global__ void __cluster_dims__(kSelBlocks, 1, 1) __launch_bounds__(kSelThreads
     const int c = blockIdx.x / kSelBlocks, part = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long n = st->n.finite > 0 ? sampling(st->n.finite).n : 0;
+    if (part == 0 && threadIdx.x == 0) st->box_min[c] = 0xffffffffu, st->box_max[c] = 0u;
     if (n == 0) {  // no finite row: an empty box (every block of the cluster leaves)
         if (part == 0 && threadIdx.x == 0) st->box_lo[c] = 1.f, st->box_hi[c] = -1.f;
         return;
@@ -492,20 +499,13 @@ __device__ __forceinline__ void row_words(const float* tile, int rows, const uin
     __syncthreads();
 }
 
-// The frame a column's moments are taken in: the middle of its box and the power of two that
-// brings its half width to about one (exact scaling, so that squares neither overflow nor vanish).
-__device__ __forceinline__ void column_frame(float2 box, float& mid, float& scale)
-{
-    mid = 0.5f * box.x + 0.5f * box.y;
-    const float half = 0.5f * box.y - 0.5f * box.x;
-    if (!isfinite(mid)) mid = 0.f;
-    int e = 0;
-    if (half > 0.f && isfinite(half)) frexpf(half, &e);
-    scale = ldexpf(1.f, -min(max(e, -100), 100));
-}
-
-// Two rows at a time in the packed float2 instructions. a + b = s + e exactly in each half (Knuth's
-// two-sum; the intrinsics keep products from being fused in).
+// The sums of a column are FP64 sums in effect: GB300's FP64 pipe (about 2 operations a clock and SM) took
+// 1.2 ms for the two passes over 2,000,003 rows, so each thread adds in three floats a row, two rows an
+// instruction in the packed float2 forms, with the rounding error of every addition carried into the
+// next word (Knuth's two-sum), and hands them to an FP64 sum every 64 rows. Against exact sums of 2 million
+// rows (normal about 0, 2 and 1e4, log-normal, uniform of size 1e-9) the relative error is at most 1.7e-15,
+// mostly that of the blocks' FP64 partial sums; all in FP64 it is up to 6.9e-15, with two words instead
+// of three 1.2e-14.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ void two_sum(float2 a, float2 b, float2& s, float2& e)
 {
@@ -513,30 +513,87 @@ __device__ __forceinline__ void two_sum(float2 a, float2 b, float2& s, float2& e
     const float2 bb = sub2(s, a);
     e = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
+struct ColumnSum {
+    static constexpr int kTiles = 4;  // of 32 rows each, between hand-overs
+    float2 h = {}, l = {}, g = {};
+    double sum = 0.0;
+    int tiles = 0;
+    __device__ __forceinline__ void low(float2 e)
+    {
+        float2 e2;
+        two_sum(l, e, l, e2);
+        g = __fadd2_rn(g, e2);
+    }
+    __device__ __forceinline__ void add(float2 x)
+    {
+        float2 e;
+        two_sum(h, x, h, e);
+        low(e);
+    }
+    __device__ __forceinline__ void hand_over()
+    {
+        sum += ((double)h.x + ((double)l.x + (double)g.x)) + ((double)h.y + ((double)l.y + (double)g.y));
+        h = l = g = make_float2(0.f, 0.f);
+        tiles = 0;
+    }
+    __device__ __forceinline__ void end_tile()
+    {
+        if (++tiles == kTiles) hand_over();
+    }
+};
 
-// keep1 (finite and inside the trim box in every column) and, over those rows, every column's
-// count, sum and sum of squares about the middle of its box. The sums are pairs of floats with the
-// rounding errors of each addition, difference and product carried along (about 46 bits), added
-// up in FP64 per block: GB300's FP64 rate (about 2 operations a clock and SM) would take 0.5 ms;
-// this takes 179 us for 2,000,003 rows, two rows an instruction (224 us one by one).
-// Four threads a column and tile; 54 x 4 of the 256 threads add.
+// The block's sum of every column (four threads each, one for 32 rows of a tile), as its own partial sum:
+// partial[block][column].
+__device__ __forceinline__ void store_partial(double (*s_sum)[kCols], ColumnSum& s, int group, int c, double* partial)
+{
+    s.hand_over();
+    if (group < 4) s_sum[group][c] = s.sum;
+    __syncthreads();
+    if (threadIdx.x < kCols)
+        partial[(long long)blockIdx.x * kCols + threadIdx.x] = (s_sum[0][threadIdx.x] + s_sum[1][threadIdx.x]) +
+                                                               (s_sum[2][threadIdx.x] + s_sum[3][threadIdx.x]);
+}
+
+// The blocks' partial sums of column c, added up by a block of 128 threads (one block for all columns
+// would take 17 us).
+__device__ __forceinline__ double column_total(const double* partial, int blocks, int c)
+{
+    __shared__ double s_sum[4];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < blocks; b += 128) s += partial[(long long)b * kCols + c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = s;
+    __syncthreads();
+    return (s_sum[0] + s_sum[1]) + (s_sum[2] + s_sum[3]);
+}
+
+// The power of two that column c's rows are added up with: 1, unless its trim box is so wide that the sum
+// could overflow.
+__device__ __forceinline__ float sum_scale(float2 box)
+{
+    return fmaxf(fabsf(box.x), fabsf(box.y)) <= 0x1p100f ? 1.f : 0x1p-40f;
+}
+
+// keep1 (finite and inside the trim box in every column) and, over those rows, every column's sum and
+// range. Four threads a column and tile; 54 x 4 of the 256 threads add.
 template <bool kVec>
 __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw, const float* __restrict__ delta,
-                                                  long long N, const uint32_t* __restrict__ finite, const Stats* __restrict__ st,
+                                                  long long N, const uint32_t* __restrict__ finite, Stats* __restrict__ st,
                                                   uint32_t* __restrict__ keep, double* __restrict__ partial,
                                                   long long* __restrict__ box_rows)
 {
     extern __shared__ __align__(16) float s_tile[];  // [2][kSubFloats], filled 16 bytes at a time
     __shared__ float2 s_box[kCols];
     __shared__ uint32_t s_part[2][4], s_words[4];
-    __shared__ double s_sum[4][kCols][2];
+    __shared__ double s_sum[4][kCols];
     for (int c = threadIdx.x; c < kCols; c += 256) s_box[c] = make_float2(st->box_lo[c], st->box_hi[c]);
     __syncthreads();
     const int c = threadIdx.x % kCols, group = threadIdx.x / kCols;  // group 4: idle
-    float mid, scale;
-    column_frame(s_box[c], mid, scale);
-    const float2 off = make_float2(-mid, -mid), sc = make_float2(scale, scale);
-    float2 h1 = {}, l1 = {}, h2 = {}, l2 = {};  // sums (high and low words) of two rows' parities
+    const float scale = sum_scale(s_box[c]);
+    const float2 sc = make_float2(scale, scale);
+    ColumnSum sum;
+    float lo = INFINITY, hi = -INFINITY;
     int kept = 0;
     for_tiles<kVec>(s_tile, raw, delta, N, [&](long long t, int rows, const float* tile) {
         row_words(tile, rows, finite, t, s_part, s_words,
@@ -551,67 +608,96 @@ __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw,
             const int step = c < kIn ? kIn : kOut;
 #pragma unroll 8
             for (int r = 0; r < 32; r += 2) {
-                // a row that is out counts as the middle: it adds exact zeros
-                const float2 v = make_float2((word >> r) & 1u ? src[r * step] : mid,
-                                             (word >> r) & 2u ? src[(r + 1) * step] : mid);
-                float2 d, e, err;
-                two_sum(v, off, d, e);
-                d = __fmul2_rn(d, sc);
-                e = __fmul2_rn(e, sc);
-                two_sum(h1, d, h1, err);
-                l1 = __fadd2_rn(l1, __fadd2_rn(err, e));
-                const float2 p = __fmul2_rn(d, d);
-                const float2 pe = __ffma2_rn(__fadd2_rn(d, d), e, __ffma2_rn(d, d, make_float2(-p.x, -p.y)));
-                two_sum(h2, p, h2, err);
-                l2 = __fadd2_rn(l2, __fadd2_rn(err, pe));
+                const float a = src[r * step], b = src[(r + 1) * step];
+                const bool in_a = (word >> r) & 1u, in_b = (word >> r) & 2u;
+                sum.add(__fmul2_rn(make_float2(in_a ? a : 0.f, in_b ? b : 0.f), sc));
+                lo = in_a ? fminf(lo, a) : lo;
+                hi = in_a ? fmaxf(hi, a) : hi;
+                lo = in_b ? fminf(lo, b) : lo;
+                hi = in_b ? fmaxf(hi, b) : hi;
             }
+            sum.end_tile();
         }
     });
-    if (group < 4) {
-        s_sum[group][c][0] = ((double)h1.x + (double)l1.x) + ((double)h1.y + (double)l1.y);
-        s_sum[group][c][1] = ((double)h2.x + (double)l2.x) + ((double)h2.y + (double)l2.y);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 2 * kCols; i += 256) {
-        const int k = i >> 1, m = i & 1;
-        partial[(long long)blockIdx.x * 2 * kCols + i] =
-            (s_sum[0][k][m] + s_sum[1][k][m]) + (s_sum[2][k][m] + s_sum[3][k][m]);
+    store_partial(s_sum, sum, group, c, partial);
+    if (group < 4 && lo <= hi) {
+        atomicMin(&st->box_min[c], float_key(lo));
+        atomicMax(&st->box_max[c], float_key(hi));
     }
     if (threadIdx.x < 4 && kept) atomicAdd(reinterpret_cast<unsigned long long*>(box_rows), (unsigned long long)kept);
 }
 
-// Mean and unbiased standard deviation of every column over the box rows (a column whose
-// deviation is below 1e-6 max(|mean|, 1) is scaled by 1) and the z limits as limits of |v - mean|.
+// Mean of every column over the box rows, and the frame of its deviations: the power of two that brings
+// the largest to between 1 and 2 (so that no square overflows, and none that counts vanishes) and the
+// mean in that scale, as the pivot that rows are taken about.
+__global__ void __launch_bounds__(128) mean_kernel(const double* __restrict__ partial, int blocks, Stats* __restrict__ st)
+{
+    const int c = blockIdx.x;
+    const double sum = column_total(partial, blocks, c);
+    if (threadIdx.x != 0) return;
+    double mean = 0.0;
+    float pivot = 0.f, scale = 1.f;
+    if (st->n.box > 0) {
+        mean = sum / (double)sum_scale(make_float2(st->box_lo[c], st->box_hi[c])) / (double)st->n.box;
+        const double far = fmax((double)key_float(st->box_max[c]) - mean, mean - (double)key_float(st->box_min[c]));
+        // to +-126, so that the power of two is a normal float
+        scale = ldexpf(1.f, far > 0.0 ? -min(max(ilogb(far), -126), 126) : 0);
+        pivot = (float)mean * scale;
+    }
+    st->mean64[c] = mean;
+    st->pivot[c] = pivot;
+    st->scale[c] = scale;
+}
+
+// Every column's sum of squared deviations from its pivot over the box rows, in its scale. A deviation is
+// a pair of floats exactly; its square goes in as the rounded product and what that leaves out.
+template <bool kVec>
+__global__ void __launch_bounds__(256) deviation_kernel(const float* __restrict__ raw, const float* __restrict__ delta,
+                                                        long long N, const uint32_t* __restrict__ box,
+                                                        const Stats* __restrict__ st, double* __restrict__ partial)
+{
+    extern __shared__ __align__(16) float s_tile[];
+    __shared__ double s_sum[4][kCols];
+    const int c = threadIdx.x % kCols, group = threadIdx.x / kCols;
+    const float2 sc = make_float2(st->scale[c], st->scale[c]);
+    const float pivot = st->pivot[c];
+    const float2 off = make_float2(-pivot, -pivot);
+    ColumnSum sum;
+    for_tiles<kVec>(s_tile, raw, delta, N, [&](long long t, int, const float* tile) {
+        if (group >= 4) return;
+        const uint32_t word = box[t * 4 + group];
+        const float* src = &tile_value(tile, 32 * group, c);
+        const int step = c < kIn ? kIn : kOut;
+#pragma unroll 8
+        for (int r = 0; r < 32; r += 2) {
+            const float2 v = __fmul2_rn(make_float2(src[r * step], src[(r + 1) * step]), sc);
+            // a row that is out counts as the pivot: it adds exact zeros
+            const float2 x = make_float2((word >> r) & 1u ? v.x : pivot, (word >> r) & 2u ? v.y : pivot);
+            float2 d, e;
+            two_sum(x, off, d, e);
+            const float2 p = __fmul2_rn(d, d);
+            sum.add(p);
+            sum.low(__ffma2_rn(__fadd2_rn(d, d), e, __ffma2_rn(d, d, make_float2(-p.x, -p.y))));
+        }
+        sum.end_tile();
+    });
+    store_partial(s_sum, sum, group, c, partial);
+}
+
+// Unbiased standard deviation of every column over the box rows (a column whose deviation is below
+// 1e-6 max(|mean|, 1) is scaled by 1) and the z limits as limits of |v - mean|. The pivot is the mean to
+// a float's rounding, 2^-24 of it, so that what the sum has to be corrected by for it is at most 2^-8 of a
+// variance that counts.
 __global__ void __launch_bounds__(128) stats_kernel(const double* __restrict__ partial, int blocks, float ood_z,
                                                     float target_clip, Stats* __restrict__ st)
 {
-    // one block a column: 65,000 FP64 additions on one SM would take 17 us
-    __shared__ double s_sum[2][4];
-    const int c = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double s[2] = {0.0, 0.0};
-    for (int b = threadIdx.x; b < blocks; b += 128) {
-        s[0] += partial[(long long)b * 2 * kCols + 2 * c];
-        s[1] += partial[(long long)b * 2 * kCols + 2 * c + 1];
-    }
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[m] += __shfl_xor_sync(0xffffffffu, s[m], o);
-        if (lane == 0) s_sum[m][warp] = s[m];
-    }
-    __syncthreads();
+    const int c = blockIdx.x;
+    const double sum = column_total(partial, blocks, c);
     if (threadIdx.x != 0) return;
-    for (int m = 0; m < 2; ++m) s[m] = (s_sum[m][0] + s_sum[m][1]) + (s_sum[m][2] + s_sum[m][3]);
     if (c < kIn) st->key_min[c] = 0xffffffffu, st->key_max[c] = 0u;
-    float mid, scale;
-    column_frame(make_float2(st->box_lo[c], st->box_hi[c]), mid, scale);
-    const double n = (double)st->n.box;
-    double mean = 0.0, sd = 0.0;
-    if (n >= 2.0) {
-        const double d = s[0] / n;
-        mean = (double)mid + d / (double)scale;
-        sd = sqrt(fmax(0.0, s[1] - s[0] * d) / (n - 1.0)) / (double)scale;
-    }
+    const double mean = st->mean64[c], n = (double)st->n.box, scale = (double)st->scale[c];
+    const double off = mean * scale - (double)st->pivot[c];
+    const double sd = n >= 2.0 ? sqrt(fmax(0.0, sum - n * off * off) / (n - 1.0)) / scale : 0.0;
     const float sf = sd > 1e-6 * fmax(fabs(mean), 1.0) ? (float)sd : 1.f;
     const float z = c < kIn ? ood_z : target_clip;
     float a = z * sf;
@@ -788,7 +874,7 @@ int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, i
     };
     const size_t at_st = place(sizeof(Stats)), at_bits = place(words * 4), at_keep = place(words * 4),
                  at_counts = place((size_t)std::max<long long>(tiles, subs) * 4),
-                 at_partial = place((size_t)blocks * 2 * kCols * 8), at_sample = place((size_t)pitch * kCols * 4);
+                 at_partial = place((size_t)blocks * kCols * 8), at_sample = place((size_t)pitch * kCols * 4);
     uint8_t* ws = nullptr;
     cudaError_t e = cudaMalloc(&ws, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "mdg_mlp_fit_normalization");
@@ -802,7 +888,8 @@ int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, i
         constexpr bool kVec = decltype(vec)::value;
         constexpr int smem = 2 * kSubFloats * (int)sizeof(float);
         cudaError_t r = cudaMemsetAsync(&d_st->n, 0, sizeof(Counts), s);
-        for (const void* f : {(const void*)box_kernel<kVec>, (const void*)zbox_kernel<kVec>, (const void*)emit_kernel<kVec>})
+        for (const void* f : {(const void*)box_kernel<kVec>, (const void*)deviation_kernel<kVec>, (const void*)zbox_kernel<kVec>,
+                              (const void*)emit_kernel<kVec>})
             if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (r != cudaSuccess) return r;
         finite_kernel<kVec><<<tiles, 256, 0, s>>>(raw, delta, N, bits, counts);
@@ -810,6 +897,8 @@ int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, i
         sample_kernel<<<tiles, 256, 0, s>>>(raw, delta, bits, counts, d_st, sample, pitch);
         select_kernel<<<kCols * kSelBlocks, kSelThreads, 0, s>>>(sample, pitch, trim_frac, margin, d_st);
         box_kernel<kVec><<<blocks, 256, smem, s>>>(raw, delta, N, bits, d_st, keep, partial, &d_st->n.box);
+        mean_kernel<<<kCols, 128, 0, s>>>(partial, blocks, d_st);
+        deviation_kernel<kVec><<<blocks, 256, smem, s>>>(raw, delta, N, keep, d_st, partial);
         stats_kernel<<<kCols, 128, 0, s>>>(partial, blocks, ood_z, target_clip, d_st);
         // the z test reads the box rows' words from `keep` and leaves the kept rows' in `bits`
         zbox_kernel<kVec><<<blocks, 256, smem, s>>>(raw, delta, N, keep, d_st, bits, counts);

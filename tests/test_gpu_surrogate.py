@@ -746,6 +746,41 @@ def test_fit_normalization_at_tile_edges(cuda, N):
     assert not x[:n, mdg.MLP_IN:].any() and not t[:n, mdg.MLP_OUT:].any() and not x[n:].any() and not t[n:].any()
 
 
+@pytest.mark.parametrize("margin", [0.0, 1e6, 1e12, 3e30, np.inf])
+def test_fit_normalization_statistics_at_any_margin(cuda, margin):
+    """Mean and deviation are taken in float64 about the mean itself, whatever the box: with wide margins
+    (a caller that does not trim), with columns far from zero against their spread, with one far row, with
+    tiny and with huge columns (the largest margins overflow, so that their limits are infinite; an infinite
+    one leaves no limit to a constant column, so none is kept). They round to float32 once (6e-8; the
+    float64 sums are good to 1e-13 of the far row's square, 1e-9 of the variance here)."""
+    N = 30007
+    rng = np.random.default_rng(7)
+    F = rng.standard_normal((N, mdg.MLP_IN + mdg.MLP_OUT))
+    F[:, 0] += 1e4
+    F[:, 1] = 1e4 + 0.05 * F[:, 1]
+    F[:, 2] *= 1e-20
+    F[:, 3] *= 1e25
+    F[N // 2, 4] = 1e3
+    if np.isfinite(margin):
+        F[:, 5] = 0.1
+    F = F.astype(np.float32)
+    raw, delta = F[:, :mdg.MLP_IN].copy(), F[:, mdg.MLP_IN:].copy()
+    m = mdg.MLP(128)
+    x = torch.zeros((N, mdg.MLP_IN_PAD), dtype=torch.bfloat16, device=cuda)
+    t = torch.zeros((N, mdg.MLP_OUT_PAD), device=cuda)
+    big = 3e38
+    counts = m.fit_normalization(torch.as_tensor(raw, device=cuda), torch.as_tensor(delta, device=cuda), x, t, trim_frac=0.0,
+                                 margin=margin, ood_z=big, target_clip=big)
+    assert counts == (N, N // 128 * 128)  # the quantiles 0 and 1 keep every row
+    K = F.astype(np.float64)
+    mean, sd = K.mean(0), K.std(0, ddof=1)
+    sd = np.where(sd > 1e-6 * np.maximum(np.abs(mean), 1.0), sd, 1.0)
+    norm = m.normalization()
+    scale = np.maximum(np.abs(mean), np.abs(K).mean(0) * 1e-6)
+    assert np.all(np.abs(np.concatenate([norm[0], norm[2]]) - mean) <= 1.2e-7 * scale)
+    np.testing.assert_allclose(np.concatenate([norm[1], norm[3]]), sd, rtol=2e-7)
+
+
 def test_fit_normalization_without_usable_rows(cuda):
     """No finite row, and a single one: refused, and the outputs stay as they were."""
     m = mdg.MLP(128)

@@ -248,6 +248,27 @@ def test_gradients_over_uneven_tile_shares(cuda, B):
 
 
 @pytest.mark.parametrize("path", [mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_MMA_SYNC])
+def test_silu_of_far_negative_pre_activations(cuda, path):
+    """SiLU is a full division in training, up to where exp(-z) overflows: with z = -88 in the whole first
+    layer h is -88 / (1 + e^88) = -5.3e-37, no zero, and the second layer's weight gradient is h times its
+    bias gradient. Both round to bf16 once (2^-9) and sum 128 rows of one sign pattern in FP32."""
+    B = 128
+    layers = [(np.array(W, np.float32), np.array(b, np.float32)) for W, b in _layers(51)]
+    layers[0][0][:], layers[0][1][:], layers[1][0][:] = 0.0, -88.0, 0.0
+    m = mdg.MLP(B, layers)
+    m.set_train_path(path)
+    x = torch.as_tensor(_inputs(52, B), device=cuda).to(torch.bfloat16)
+    t = torch.full((B, mdg.MLP_OUT_PAD), 1e10, device=cuda)
+    m.grad(x, t)
+    assert m.status() == 0
+    g = mdg.mlp_unflatten(m.grads())
+    h = -88.0 / (1.0 + np.exp(88.0))
+    want = np.outer(g[1][1], np.full(mdg.MLP_HIDDEN, h))
+    assert np.abs(want).max() > 1e-35
+    np.testing.assert_allclose(g[1][0], want, rtol=2.0 ** -7, atol=2.0 ** -7 * np.abs(want).max())
+
+
+@pytest.mark.parametrize("path", [mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_MMA_SYNC])
 def test_loss_at_any_address(cuda, path):
     """The loss goes to any address that a copy can reach: one that is not 4-byte aligned (no kernel
     stores to it) receives the same four bytes, and its neighbours stay as they were."""

@@ -70,7 +70,8 @@ __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 
-// 1 / x for normal x: the approximation and a Newton step, to about half an ulp.
+// 1 / x, correctly rounded, where x and the result are normal: the approximation and a Newton step (equal to
+// the division for all 2^23 mantissas).
 __device__ __forceinline__ float rcp_newton(float x)
 {
     const float r = rcp_approx(x);
@@ -264,7 +265,10 @@ __global__ void __launch_bounds__(kCamThreads) render_kernel(const CamArgs a)
     // the largest ray parameter for which both ground coordinates stay within 2^20 m (floor2), from
     // bounds of the origin and of the ray's horizontal components
     const float span = fmaxf(fabsf(C.m[0]) + fabsf(C.m[1]) + fabsf(C.m[2]), fabsf(C.m[3]) + fabsf(C.m[4]) + fabsf(C.m[5]));
-    const float reach = fabsf(ox) < 262144.f && fabsf(oy) < 262144.f ? 262144.f / fmaxf(span, 1.f) : 0.f;
+    // (none, 0, where the slopes' reciprocals may leave the range of rcp_newton)
+    const float rise = fabsf(C.m[6]) + fabsf(C.m[7]) + fabsf(C.m[8]);
+    const uint32_t reach = __float_as_uint(
+        fabsf(ox) < 262144.f && fabsf(oy) < 262144.f && rise < 0x1p120f ? 262144.f / fmaxf(span, 1.f) : 0.f);
     for (int tx = kWarp ? 0 : t >> 5; tx < (kWarp ? kTilesX : (t >> 5) + 1); ++tx) {
         const int col = tx * kTileW + (lane & 3) * kPx;
         // world direction of the body ray (1, -nx, ny), not normalised: its component along
@@ -296,14 +300,14 @@ __global__ void __launch_bounds__(kCamThreads) render_kernel(const CamArgs a)
             }
             // the ground: d2 is linear along the row, so the ends tell whether any pixel looks down
             if (above && fminf(d2[0], d2[kPx - 1]) < 0.f) {
-                float far = 0.f;
+                uint32_t far = 0;  // bits of the farthest hit (a NaN counts as farther than any)
                 bool down[kPx];
 #pragma unroll
                 for (int i = 0; i < kPx; ++i) {
                     const float tg = -oz * rcp_newton(d2[i]);
-                    down[i] = d2[i] < 0.f && tg > kTMin;
+                    down[i] = d2[i] < 0.f && !(tg <= kTMin);
                     t_best[i] = down[i] ? tg : kInf;
-                    far = fmaxf(far, down[i] ? tg : 0.f);
+                    far = max(far, down[i] ? __float_as_uint(tg) : 0u);
                     seg[i] = down[i] ? 0 : -1;
                 }
                 if (far < reach) {
@@ -313,11 +317,15 @@ __global__ void __launch_bounds__(kCamThreads) render_kernel(const CamArgs a)
                         const uint32_t odd = floor2(fmaf(tg, d0[i], ox)) ^ floor2(fmaf(tg, d1[i], oy));
                         color[i] = down[i] ? ((odd & 1u) ? c_dark : c_light) : c_sky;
                     }
-                } else {  // close to the horizon
+                } else {  // close to the horizon: by the division itself, which takes any slope
 #pragma unroll
                     for (int i = 0; i < kPx; ++i) {
-                        if (!down[i]) continue;
-                        const float px = fmaf(t_best[i], d0[i], ox), py = fmaf(t_best[i], d1[i], oy);
+                        const float tg = d2[i] < 0.f ? -oz * (1.f / d2[i]) : 0.f;
+                        const bool hits = tg > kTMin;
+                        t_best[i] = hits ? tg : kInf;
+                        seg[i] = hits ? 0 : -1;
+                        if (!hits) continue;
+                        const float px = fmaf(tg, d0[i], ox), py = fmaf(tg, d1[i], oy);
                         const int odd = (int)floorf(px * 2.f) + (int)floorf(py * 2.f);
                         color[i] = (odd & 1) ? c_dark : c_light;
                     }

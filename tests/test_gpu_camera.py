@@ -154,3 +154,23 @@ def test_warp_and_block_forms_and_unaligned_outputs_agree(cuda):
     assert np.all(np.isfinite(depth[ground])) and np.all(np.isinf(depth[seg == -1]))
     greys = {tuple(c) for c in rgba[ground][:, :3]}
     assert len(greys) == 2 and not ground[2].any()  # two greys; nothing seen from below
+
+
+@pytest.mark.parametrize("drones", [1, 33])
+def test_rays_almost_along_the_ground(cuda, drones):
+    """Rays whose slope is not a normal float meet the ground where they fall, farther away than a float
+    can say, and the sky where they rise: a camera whose attitude leaves it slopes of 1e-39 either way."""
+    p = np.zeros((drones, 3), np.float32)
+    p[:, 0], p[:, 2] = -30.0 * np.arange(drones), 1.0  # the others are behind the camera
+    q = np.zeros((drones, 4), np.float32)
+    w, z = 1e-39, 0.8e-39
+    q[0], q[1:, 0] = (w, 0.5, 0.5, z), 1.0  # 1 - 2 (x^2 + y^2) = 0, 2 (xz - wy) = z - w, 2 (yz + wx) = z + w
+    v = np.zeros((drones, 3), np.float32)
+    h = mdg.Handle([drones], [0])
+    rgba, depth, seg = h.new_frames(cuda)
+    h.render(mdg.pack_state(p, q, v, v, device=cuda), rgba, depth, seg)
+    nx = ((np.arange(mdg.CAM_W) + 0.5) * (2 / mdg.CAM_W) - 1) * np.tan(np.pi / 6) * mdg.CAM_W / mdg.CAM_H
+    down = np.broadcast_to((z - w) - nx * (z + w) < 0, (mdg.CAM_H, mdg.CAM_W))
+    assert down.any() and not down.all()
+    np.testing.assert_array_equal(seg[0].cpu().numpy(), np.where(down, 0, -1))
+    assert torch.all(depth[0] > 1e38)

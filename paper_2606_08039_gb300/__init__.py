@@ -231,21 +231,20 @@ def _ptr(t, name, dtype, shape=None):
     """Address of a contiguous CUDA tensor of the given type and shape (None: no tensor)."""
     if t is None:
         return None
-    try:
-        if t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
-            return t.data_ptr()
-    except AttributeError:
-        pass
-    torch = _torch()
+    torch = _torch_module or _torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous() and (shape is None or t.shape == shape):
+        return t.data_ptr()
     if t.device.type != "cuda":
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+    if shape is not None and tuple(t.shape) != tuple(shape):
+        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+    return t.data_ptr()
 
 
 def _host_ptr(t, name, dtype, shape=None):

@@ -191,3 +191,23 @@ def test_dynamic_shared_memory_is_declared_aligned():
                 assert decl.startswith("float4 ") or (align and int(align.group(1)) >= 16), f"{name}: {decl}"
                 found += 1
     assert found >= 10
+
+
+def test_only_tensors_are_marshalled():
+    """An object that looks like a CUDA tensor but is none is refused, as any other argument that is no tensor."""
+    torch = pytest.importorskip("torch")
+
+    class Lookalike:
+        is_cuda, dtype, shape = True, torch.float32, (4,)
+
+        def is_contiguous(self):
+            return True
+
+        def data_ptr(self):
+            return 16
+    for t in (Lookalike(), np.zeros(4, np.float32), 16):
+        with pytest.raises(TypeError, match="x must be a torch tensor"):
+            mdg._ptr(t, "x", torch.float32, (4,))
+    with pytest.raises(ValueError, match="x must be a CUDA tensor"):
+        mdg._ptr(torch.zeros(4), "x", torch.float32, (4,))
+    assert mdg._ptr(None, "x", torch.float32, (4,)) is None

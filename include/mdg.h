@@ -462,7 +462,8 @@ int mdg_get_rollout_schedule(mdg_handle h, int32_t* mode, int32_t* item_drones);
  * both schedules of mdg_set_rollout_schedule and (uneven batches) the item caps of the whole
  * block, half and a quarter of it (at least the largest environment and 32 drones): 5 timed
  * launches after 2 warm-ups each, the state restored before every launch. Keeps the fastest
- * combination (mdg_set_block_size, mdg_set_rollout_schedule) and restores the state.
+ * combination (mdg_set_block_size, mdg_set_rollout_schedule) and restores the state. (K = 0
+ * for randomized steps that always take blocks of 64 drones: the handle's block size stays.)
  * Allocates temporary scratch; synchronises `stream`. Writes the chosen block size and its
  * mean time in ms (either pointer may be NULL; mdg_get_rollout_schedule reads the rest). */
 int mdg_autotune(mdg_handle h, float* state, const float* actions, int32_t action_per_step, int32_t action_type,

@@ -1287,7 +1287,11 @@ int mdg_autotune(mdg_handle h, float* state, const float* actions, int32_t actio
             int block, sched, cap;
         };
         std::vector<Cand> cands;
-        for (int b = lo; b <= 1024; b = b < 64 ? 64 : b * 2) {
+        // a step whose blocks are of one size whatever the handle's keeps the handle's: all candidates would
+        // launch alike, and chance would choose the block of the rollouts and observations
+        const bool one_size = K == 0 && h->dr && mdg::draws_apart(h->uniform_N);
+        if (one_size) cands.push_back({original, orig_sched, orig_cap});
+        for (int b = lo; b <= 1024 && !one_size; b = b < 64 ? 64 : b * 2) {
             if (K == 0) {
                 cands.push_back({b, orig_sched, orig_cap});
                 continue;

@@ -247,6 +247,9 @@ inline bool valid_action(int t) { return valid_env_action(t) || t == MDG_ACT_MIX
 inline bool extended_action(int t) { return t >= MDG_ACT_RPM_NORM && t <= MDG_ACT_ATTITUDE; }
 // grid: persistent CTAs (0: one per work item)
 cudaError_t launch_rollout(const RolloutArgs& a, int block, int uniform_flags, int grid, cudaStream_t s);
+// Whether randomized steps of environments of one size (0: of several) take the kernel with a drawing warp,
+// whose blocks are of one size whatever the handle's.
+inline bool draws_apart(int uniform_N) { return uniform_N > 0 && uniform_N <= 32; }
 int rollout_blocks_per_sm(const StepArgs& a, int block, int uniform_flags);
 cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s);
 // mdg_surrogate.cu: mdg_features of the RPMs rpm (times rpm_scale, when given), which go to applied

@@ -2425,7 +2425,7 @@ cudaError_t launch_step(const StepArgs& a, int n_tiles, int block, bool with_obs
     // batch) and per-rotor ground heights run in runtime-flag variants of their own
     int flags, N;
     variant_of(a, uniform_flags, flags, N);
-    if (flags == kFlagsDR && N > 0 && N <= 32) {
+    if (flags == kFlagsDR && draws_apart(N)) {
         StepArgs r = a;
         r.envs_per_tile = kDrawDrones / N;
         bool local = true;

@@ -296,3 +296,18 @@ def test_step_kernels_agree_with_the_rollout(cuda, drones, envs, depth):
     assert torch.equal(a[4].isnan(), b[4].isnan()) and torch.equal(a[-1], b[-1])
     for name, x, y in zip(("state", "kin", "rel", "motor", "history", "wind"), a, b):
         np.testing.assert_allclose(x.cpu().numpy(), y.cpu().numpy(), rtol=1e-5, atol=1e-5, err_msg=name)
+
+
+def test_autotune_keeps_the_block_where_the_step_has_its_own(cuda):
+    """Randomized steps of up to 32 drones per environment take blocks of 64 drones whatever the handle's
+    size: tuning them leaves the size that rollouts and observations use."""
+    sw = wl.full_aero(211, n_envs=64, drones=4)
+    h = mdg.Handle(sw.drones_per_env, sw.flags)
+    live = h.new_randomization_state(3, cuda)
+    h.set_randomization(torch.as_tensor(wl.dr_table(212, 64, depth=3), device=cuda), *live, seed=SEED)
+    state = mdg.pack_state(sw.p, sw.q, sw.v, sw.w, device=cuda)
+    act = torch.as_tensor(wl.waypoints(213, sw.n), device=cuda)
+    for block in (32, 128, 256, 1024):
+        h.set_block_size(block)
+        best, ms = h.autotune(state, act, mdg.ACT_PID, 5, 0)
+        assert best == h.block_size == block and ms > 0

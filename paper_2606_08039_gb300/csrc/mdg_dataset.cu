@@ -22,6 +22,7 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kIn = MDG_MLP_IN, kOut = MDG_MLP_OUT, kCols = kIn + kOut;
+static_assert(kCols % 6 == 0, "the sample's rounds of six columns");
 constexpr int kTile = 1024;  // rows of one block of the finite test and the sampling
 constexpr int kSampleMax = 262144;
 
@@ -224,13 +225,14 @@ __device__ __forceinline__ Sampling sampling(long long n_finite)
     return s;
 }
 
-// Copies the sampled rows, as float keys, column by column: sample[c * pitch + s]. Rows are read
-// whole and turned in shared memory (a pitch of 55 words: no bank conflict either way).
+// Copies `cols` columns from c0 of the sampled rows, as float keys, column by column:
+// sample[(c - c0) * pitch + s]. Rows are read whole and turned in shared memory (a pitch of 55
+// words: no bank conflict either way).
 constexpr int kSampleRows = 128;
 __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ raw, const float* __restrict__ delta,
                                                      const uint32_t* __restrict__ bits, const int* __restrict__ offsets,
-                                                     const Stats* __restrict__ st, uint32_t* __restrict__ sample,
-                                                     long long pitch)
+                                                     const Stats* __restrict__ st, int c0, int cols,
+                                                     uint32_t* __restrict__ sample, long long pitch)
 {
     __shared__ int s_row[kTile];  // tile row of each sampled row
     __shared__ uint32_t s_keys[kSampleRows][kCols + 1];
@@ -267,8 +269,8 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ r
             if (lane < kCols - 32) s_keys[k][32 + lane] = float_key(column(raw, delta, r, 32 + lane));
         }
         __syncthreads();
-        for (int c = warp; c < kCols; c += 8)
-            for (int k = lane; k < m; k += 32) sample[c * pitch + first + k0 + k] = s_keys[k][c];
+        for (int c = warp; c < cols; c += 8)
+            for (int k = lane; k < m; k += 32) sample[c * pitch + first + k0 + k] = s_keys[k][c0 + c];
         __syncthreads();
     }
 }
@@ -283,14 +285,14 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ r
 // block a column took 230 us, clusters of eight 194 us.
 constexpr int kSelBlocks = 4, kSelThreads = 512;
 __global__ void __cluster_dims__(kSelBlocks, 1, 1) __launch_bounds__(kSelThreads, 2)
-    select_kernel(const uint32_t* __restrict__ sample, long long pitch, float trim_frac, float margin,
+    select_kernel(const uint32_t* __restrict__ sample, long long pitch, int c0, float trim_frac, float margin,
                   Stats* __restrict__ st)
 {
     __shared__ unsigned s_hist[4][2048];
     __shared__ uint32_t s_prefix[4];
     __shared__ unsigned s_rank[4];
     cg::cluster_group cluster = cg::this_cluster();
-    const int c = blockIdx.x / kSelBlocks, part = (int)cluster.block_rank();
+    const int c = c0 + blockIdx.x / kSelBlocks, part = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long n = st->n.finite > 0 ? sampling(st->n.finite).n : 0;
     if (part == 0 && threadIdx.x == 0) st->box_min[c] = 0xffffffffu, st->box_max[c] = 0u;
@@ -305,7 +307,7 @@ __global__ void __cluster_dims__(kSelBlocks, 1, 1) __launch_bounds__(kSelThreads
         s_prefix[threadIdx.x] = 0;
     }
     // this block's quarter, in 16-byte pieces; the last block also takes the keys beyond whole pieces
-    const uint32_t* key = sample + c * pitch;
+    const uint32_t* key = sample + (c - c0) * pitch;
     const uint4* key4 = reinterpret_cast<const uint4*>(key);
     const int n4 = (int)(n / 4), per = (n4 + kSelBlocks - 1) / kSelBlocks;
     const int i0 = min(n4, part * per), i1 = min(n4, i0 + per);
@@ -865,18 +867,34 @@ int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, i
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int blocks = (int)std::min<long long>(subs, 4LL * n_sm);
-    // one allocation, carved up
-    size_t bytes = 0;
-    auto place = [&bytes](size_t n) {
-        const size_t at = bytes;
-        bytes += (n + 255) / 256 * 256;
-        return at;
-    };
-    const size_t at_st = place(sizeof(Stats)), at_bits = place(words * 4), at_keep = place(words * 4),
-                 at_counts = place((size_t)std::max<long long>(tiles, subs) * 4),
-                 at_partial = place((size_t)blocks * kCols * 8), at_sample = place((size_t)pitch * kCols * 4);
+    // one allocation, carved up: with the sample of all columns, or of six, or of one at a time where
+    // there is no room for it (113 MB of it above half a million rows)
+    size_t at_st = 0, at_bits = 0, at_keep = 0, at_counts = 0, at_partial = 0, at_sample = 0;
     uint8_t* ws = nullptr;
-    cudaError_t e = cudaMalloc(&ws, bytes);
+    int cols = kCols;
+    cudaError_t e;
+    for (;;) {
+        size_t bytes = 0;
+        auto place = [&bytes](size_t n) {
+            const size_t at = bytes;
+            bytes += (n + 255) / 256 * 256;
+            return at;
+        };
+        at_st = place(sizeof(Stats));
+        at_bits = place(words * 4);
+        at_keep = place(words * 4);
+        at_counts = place((size_t)std::max<long long>(tiles, subs) * 4);
+        at_partial = place((size_t)blocks * kCols * 8);
+        at_sample = place((size_t)pitch * cols * 4);
+#ifdef MDG_DEBUG
+        e = cols == kCols ? cudaErrorMemoryAllocation : cudaMalloc(&ws, bytes);  // as if there were no room
+#else
+        e = cudaMalloc(&ws, bytes);
+#endif
+        if (e != cudaErrorMemoryAllocation || cols == 1) break;
+        cudaGetLastError();
+        cols = cols > 6 ? 6 : 1;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "mdg_mlp_fit_normalization");
     Stats* d_st = reinterpret_cast<Stats*>(ws + at_st);
     uint32_t *bits = reinterpret_cast<uint32_t*>(ws + at_bits), *keep = reinterpret_cast<uint32_t*>(ws + at_keep);
@@ -894,8 +912,10 @@ int mdg_mlp_fit_normalization(mdg_mlp m, const float* raw, const float* delta, i
         if (r != cudaSuccess) return r;
         finite_kernel<kVec><<<tiles, 256, 0, s>>>(raw, delta, N, bits, counts);
         scan_kernel<<<1, 1024, 0, s>>>(counts, tiles, &d_st->n.finite);
-        sample_kernel<<<tiles, 256, 0, s>>>(raw, delta, bits, counts, d_st, sample, pitch);
-        select_kernel<<<kCols * kSelBlocks, kSelThreads, 0, s>>>(sample, pitch, trim_frac, margin, d_st);
+        for (int c = 0; c < kCols; c += cols) {
+            sample_kernel<<<tiles, 256, 0, s>>>(raw, delta, bits, counts, d_st, c, cols, sample, pitch);
+            select_kernel<<<cols * kSelBlocks, kSelThreads, 0, s>>>(sample, pitch, c, trim_frac, margin, d_st);
+        }
         box_kernel<kVec><<<blocks, 256, smem, s>>>(raw, delta, N, bits, d_st, keep, partial, &d_st->n.box);
         mean_kernel<<<kCols, 128, 0, s>>>(partial, blocks, d_st);
         deviation_kernel<kVec><<<blocks, 256, smem, s>>>(raw, delta, N, keep, d_st, partial);

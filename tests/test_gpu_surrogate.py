@@ -2,6 +2,11 @@
 oracle (forward, gradients, Adam), its inputs against the dynamics oracle, and the
 surrogate control step: its one-step error against the plain integrator, what the network
 gains over predicting no change, and the out-of-distribution fallback."""
+import hashlib
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -16,6 +21,7 @@ from helpers import assert_horizon_close, assert_knn_valid, check_obs_against_ow
 
 pytestmark = pytest.mark.gpu
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 P = oracle.cf2x()
 HOVER = oracle.hover_rpm(P)
 
@@ -800,6 +806,35 @@ def test_fit_normalization_statistics_at_any_margin(cuda, margin):
     scale = np.maximum(np.abs(mean), np.abs(K).mean(0) * 1e-6)
     assert np.all(np.abs(np.concatenate([norm[0], norm[2]]) - mean) <= 1.2e-7 * scale)
     np.testing.assert_allclose(np.concatenate([norm[1], norm[3]]), sd, rtol=2e-7)
+
+
+def _fit_digest(cuda):
+    """Digest of what fit_normalization returns for a set below and one above the sample's first stride."""
+    digest = hashlib.sha256()
+    for N in (5003, 600001):
+        g = torch.Generator(device=cuda)
+        g.manual_seed(N)
+        F = torch.randn((N, mdg.MLP_IN + mdg.MLP_OUT), generator=g, device=cuda)
+        m = mdg.MLP(128)
+        x = torch.zeros((N, mdg.MLP_IN_PAD), dtype=torch.bfloat16, device=cuda)
+        t = torch.zeros((N, mdg.MLP_OUT_PAD), device=cuda)
+        counts = m.fit_normalization(F[:, :mdg.MLP_IN].contiguous(), F[:, mdg.MLP_IN:].contiguous(), x, t)
+        for a in (np.array(counts), *m.normalization(), x.view(torch.int16).cpu().numpy(), t.cpu().numpy()):
+            digest.update(np.ascontiguousarray(a).tobytes())
+    return digest.hexdigest()
+
+
+def test_fit_normalization_with_a_small_workspace(cuda):
+    """Where the sample of all columns finds no room it is taken a few columns at a time, with the same
+    result bit for bit. The debug build takes the first workspace as refused."""
+    from paper_2606_08039_gb300 import build
+    build.build_library(debug=True)
+    code = ("import sys; sys.path.insert(0, 'tests'); import torch; import test_gpu_surrogate as t; "
+            "assert t.mdg.LIB_PATH.endswith('libmdg_debug.so'); print('digest', t._fit_digest(torch.device('cuda', 0)))")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, MDG_DEBUG_LIBRARY="1", PYTHONPATH=ROOT),
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-3000:]
+    assert r.stdout.split()[-1] == _fit_digest(cuda)
 
 
 def test_fit_normalization_without_usable_rows(cuda):

@@ -253,6 +253,35 @@ def test_gradients_over_uneven_tile_shares(cuda, B):
     test_gradients_and_loss_match_oracle(cuda, mdg.MLP_PATH_TCGEN05, B)
 
 
+def test_weight_gradients_of_a_large_batch(cuda):
+    """The output layer's gradients of 131072 rows, whose sums grow without cancelling, against the same
+    network in float64 with the same bf16 roundings. Activations near a bf16 rounding boundary flip on one
+    side (about 1e-4 of them, by 2^-8: 1e-7 over the batch); the tensor cores cut FP32 sums off by up to
+    2^-24 every 16 rows, 48 times in a run, 3e-6; the additions of 171 runs round to 2^-24 each, 1e-6."""
+    B = 131072
+    layers = _layers(61)
+    m = mdg.MLP(B, layers)
+    g = torch.Generator(device=cuda)
+    g.manual_seed(62)
+    x = torch.zeros((B, mdg.MLP_IN_PAD), device=cuda)
+    x[:, :mdg.MLP_IN] = torch.randn((B, mdg.MLP_IN), generator=g, device=cuda)
+    x = x.bfloat16()
+    t = torch.full((B, mdg.MLP_OUT_PAD), 4.0, device=cuda)
+    m.grad(x, t)
+    assert m.status() == 0
+    W4, b4 = mdg.mlp_unflatten(m.grads())[3]
+    h = x.double()
+    for l in range(4):
+        W, b = (torch.as_tensor(np.asarray(a, np.float32), device=cuda) for a in layers[l])
+        z = h @ W.bfloat16().double().T + b.double()
+        h = (z * torch.sigmoid(z)).float().bfloat16().double() if l < 3 else h
+    d = (z - t.double()) * (torch.arange(mdg.MLP_OUT_PAD, device=cuda) < mdg.MLP_OUT)
+    dy = (d * (2 / (B * mdg.MLP_OUT))).float().bfloat16().double()
+    for got, want in ((W4, dy.T @ h), (b4, dy.sum(0))):
+        got = torch.as_tensor(got, device=cuda).double()
+        assert float((got - want).norm() / want.norm()) < 5e-6
+
+
 @pytest.mark.parametrize("path", [mdg.MLP_PATH_TCGEN05, mdg.MLP_PATH_MMA_SYNC])
 def test_silu_of_far_negative_pre_activations(cuda, path):
     """SiLU is a full division in training, up to where exp(-z) overflows: with z = -88 in the whole first

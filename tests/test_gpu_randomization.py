@@ -258,13 +258,15 @@ def test_obs_bias_needs_randomization(cuda):
         h.set_obs_bias(torch.zeros((sw.n, 12), device=cuda))
 
 
-@pytest.mark.parametrize("drones,envs,depth", [(1, 70, 1), (2, 33, 2), (3, 43, 4), (4, 17, 3), (5, 13, 5), (31, 5, 3),
-                                               (32, 3, 3), (33, 3, 3)])
-def test_step_kernels_agree_with_the_rollout(cuda, drones, envs, depth):
+@pytest.mark.parametrize("block", [None, 512])
+@pytest.mark.parametrize("drones,envs,depth", [(1, 70, 1), (2, 33, 2), (3, 43, 4), (4, 17, 3), (5, 13, 5), (8, 9, 2),
+                                               (16, 5, 3), (31, 5, 3), (32, 3, 3), (33, 3, 3)])
+def test_step_kernels_agree_with_the_rollout(cuda, drones, envs, depth, block):
     """Three randomized control steps one by one (uniform batches of up to 32 drones: the kernel with
     a drawing warp; 33: the general one) against the same steps as one rollout, whose drones draw
     for themselves: partial blocks, environments across warps, histories of 1 to 5 rows, every
-    action type. The same float32 formulas in another order of noise and bias: heights are spread,
+    action type. In blocks of 512 the rollout reads the downwash sources one by one, where the steps of
+    even sizes inside a warp read them in pairs. The same float32 formulas in another order of noise and bias: heights are spread,
     so 15 substeps amplify a rounding (6e-8) by far less than the 100 that 1e-5 allows; the rotor
     speeds (to 2e4), histories and step counters alike."""
     sw = spread_heights(wl.full_aero(201, n_envs=envs, drones=drones))
@@ -276,6 +278,8 @@ def test_step_kernels_agree_with_the_rollout(cuda, drones, envs, depth):
     got = []
     for rollout in (False, True):
         h = mdg.Handle(sw.drones_per_env, sw.flags)
+        if rollout and block:
+            h.set_block_size(block)
         h.set_action_types(types)
         live = h.new_randomization_state(depth, cuda)
         h.set_randomization(torch.as_tensor(table, device=cuda), *live, seed=SEED)

@@ -74,6 +74,30 @@ def test_variants_agree(cuda, drones, rk4):
                              what=f"{drones} drones")
 
 
+@pytest.mark.parametrize("rk4", [False, True])
+@pytest.mark.parametrize("sizes", [[10] * 7, [12] * 9, [14] * 5, [18] * 4, [30] * 3, [6, 10, 16, 1, 1, 2, 8, 12, 32, 14, 18]])
+def test_runtime_pairs_agree_with_single_sources(cuda, sizes, rk4):
+    """Even sizes without a variant of their own, at even places inside the warps of small blocks, read the
+    downwash sources in pairs; the same environments in blocks of 512 read them one by one."""
+    dpe = np.array(sizes, np.int32)
+    place = 0
+    for n in sizes:  # as whole environments fill blocks of 32 drones
+        place = 0 if place + n > 32 else place
+        assert n == 1 or (place % 2 == 0 and n % 2 == 0)
+        place += n
+    n = int(dpe.sum())
+    p = np.zeros((n, 3), np.float32)
+    k = np.concatenate([np.arange(m) for m in sizes])
+    p[:, 0], p[:, 1], p[:, 2] = 0.3 * (k % 4), 0.3 * (k // 4), 0.4 + 0.2 * k  # every drone on a height of its own
+    _, q, v, w = wl.random_states(303, n)
+    sw = (p, q, 0.1 * v, 0.1 * w)
+    runs = [_run(cuda, dpe, sw, rk4, r, b) for b in (32, 512) for r in (False, True)]
+    for other in runs[1:]:
+        assert torch.equal(runs[0][2], other[2])
+        for a, b in zip((runs[0][0], runs[0][1], runs[0][3]), (other[0], other[1], other[3])):
+            torch.testing.assert_close(a, b, rtol=1e-5, atol=1e-5)
+
+
 def _rk4_constants():
     c = mdg.Constants.cf2x()
     c.integrator = mdg.INTEGRATOR_RK4

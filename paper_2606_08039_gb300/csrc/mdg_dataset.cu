@@ -811,8 +811,6 @@ __global__ void __launch_bounds__(256) emit_kernel(const float* __restrict__ raw
     });
 }
 
-int grid_for(long long n, int block) { return (int)std::min<long long>((n + block - 1) / block, 152 * 16); }
-
 }  // namespace
 
 extern "C" {

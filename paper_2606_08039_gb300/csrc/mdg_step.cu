@@ -11,8 +11,6 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
-#include <initializer_list>
-
 #include "mdg.h"
 #include "mdg_internal.cuh"
 

@@ -319,7 +319,8 @@ cudaError_t upload(T** dst, const std::vector<T>& v)
 
 // The dependent chain of one substep of an environment of N drones, in units of the
 // instructions of a substep without downwash (~160), for the static schedule: the drones of
-// a work item run in parallel threads, so an item lasts about as long as its longest chain.
+// a work item run in parallel threads, so an item lasts about as long as its longest chain. (23 a
+// source is the single sources' loop; the packed one of kPaired batches takes 16.)
 double item_chain(int N, uint32_t flags) { return 160.0 + ((flags & MDG_DW) ? 23.0 * (N - 1) : 0.0); }
 
 // Work items of the rollout kernel for the current block size and item cap. Uniform batches

@@ -1390,8 +1390,8 @@ __device__ __forceinline__ void rk4_substeps(Drone& d, const Motor& m, const Env
     }
 }
 
-// Variants with a compile-time environment size (kN > 0), and the runtime-size variant
-// kN = -1, run blocks of at most kSmallBlock threads and may use up to 128 registers;
+// Variants with a compile-time environment size (kN > 0), and the runtime-size variants
+// kN = -1 and -2, run blocks of at most kSmallBlock threads and may use up to 128 registers;
 // the kN = 0 variant takes any block size (64 registers).
 constexpr int kSmallBlock = 256;
 template <int kN>

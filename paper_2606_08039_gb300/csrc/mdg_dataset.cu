@@ -570,12 +570,8 @@ __device__ __forceinline__ double column_total(const double* partial, int blocks
     return (s_sum[0] + s_sum[1]) + (s_sum[2] + s_sum[3]);
 }
 
-// The power of two that column c's rows are added up with: 1, unless its trim box is so wide that the sum
-// could overflow.
-__device__ __forceinline__ float sum_scale(float2 box)
-{
-    return fmaxf(fabsf(box.x), fabsf(box.y)) <= 0x1p100f ? 1.f : 0x1p-40f;
-}
+// Bound of a trim box within which no run of 64 rows overflows; wider columns are added in FP64 as they are.
+constexpr float kHuge = 0x1p100f;
 
 // keep1 (finite and inside the trim box in every column) and, over those rows, every column's sum and
 // range. Four threads a column and tile; 54 x 4 of the 256 threads add.
@@ -592,8 +588,7 @@ __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw,
     for (int c = threadIdx.x; c < kCols; c += 256) s_box[c] = make_float2(st->box_lo[c], st->box_hi[c]);
     __syncthreads();
     const int c = threadIdx.x % kCols, group = threadIdx.x / kCols;  // group 4: idle
-    const float scale = sum_scale(s_box[c]);
-    const float2 sc = make_float2(scale, scale);
+    const bool wide = !(fmaxf(fabsf(s_box[c].x), fabsf(s_box[c].y)) <= kHuge);
     ColumnSum sum;
     float lo = INFINITY, hi = -INFINITY;
     int kept = 0;
@@ -608,15 +603,23 @@ __global__ void __launch_bounds__(256) box_kernel(const float* __restrict__ raw,
             const uint32_t word = s_words[group];
             const float* src = &tile_value(tile, 32 * group, c);
             const int step = c < kIn ? kIn : kOut;
+            auto row = [&](int r, float& v) {
+                v = src[r * step];
+                const bool in = (word >> r) & 1u;
+                lo = in ? fminf(lo, v) : lo;
+                hi = in ? fmaxf(hi, v) : hi;
+                v = in ? v : 0.f;
+            };
+            float2 x;
+            if (wide) {
+                for (int r = 0; r < 32; ++r) row(r, x.x), sum.sum += (double)x.x;
+            } else {
 #pragma unroll 8
-            for (int r = 0; r < 32; r += 2) {
-                const float a = src[r * step], b = src[(r + 1) * step];
-                const bool in_a = (word >> r) & 1u, in_b = (word >> r) & 2u;
-                sum.add(__fmul2_rn(make_float2(in_a ? a : 0.f, in_b ? b : 0.f), sc));
-                lo = in_a ? fminf(lo, a) : lo;
-                hi = in_a ? fmaxf(hi, a) : hi;
-                lo = in_b ? fminf(lo, b) : lo;
-                hi = in_b ? fmaxf(hi, b) : hi;
+                for (int r = 0; r < 32; r += 2) {
+                    row(r, x.x);
+                    row(r + 1, x.y);
+                    sum.add(x);
+                }
             }
             sum.end_tile();
         }
@@ -640,7 +643,7 @@ __global__ void __launch_bounds__(128) mean_kernel(const double* __restrict__ pa
     double mean = 0.0;
     float pivot = 0.f, scale = 1.f;
     if (st->n.box > 0) {
-        mean = sum / (double)sum_scale(make_float2(st->box_lo[c], st->box_hi[c])) / (double)st->n.box;
+        mean = sum / (double)st->n.box;
         const double far = fmax((double)key_float(st->box_max[c]) - mean, mean - (double)key_float(st->box_min[c]));
         // to +-126, so that the power of two is a normal float
         scale = ldexpf(1.f, far > 0.0 ? -min(max(ilogb(far), -126), 126) : 0);

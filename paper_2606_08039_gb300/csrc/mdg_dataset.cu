@@ -102,11 +102,11 @@ __host__ __device__ inline float key_float(uint32_t k)
 // and 256 B a row written. Every number that a later kernel needs stays on the device, so the host
 // waits once, at the end. 2,000,003 rows: 7.1 ms with a thread per row or per element (32 counting
 // passes for the quantiles, FP64 shared-memory atomics for the moments, 15 allocations and 8
-// waits), 1.1 ms now: finite 74 us (5.8 TB/s), sample 58, selection 97, box and sums 144, deviations
+// waits), 1.1 ms now: finite 74 us (5.8 TB/s), sample 58, selection 97, box and sums 140, deviations
 // 157 (both their arithmetic), z limits 76 (5.7 TB/s), training set 141 (5.9 TB/s, both ways), the
 // two scans, means and statistics 35; the rest is the one allocation and its release (150 us) and
 // the host's copies. (One pass for sum and square about the middle of the box took 179 us instead of
-// the 301 of two, but lost deviations to cancellation and overflow where the box is wide: without a
+// the 297 of two, but lost deviations to cancellation and overflow where the box is wide: without a
 // limit, margin = inf, one of 0.05 about 1e4 came out 8e-5 of itself off and a column of size 1e25 as constant.)
 
 // Counts of the set: finite rows, rows inside the trim box, rows kept.

@@ -405,18 +405,11 @@ cudaError_t launch_render(const CamArgs& a, cudaStream_t s)
     const bool warp = a.max_env <= 32;
     const int teams = warp ? kCamThreads / 32 : 1;
     const int smem = teams * a.max_env * kSceneF4 * (int)sizeof(float4);
-    if (smem > 48 * 1024) {  // the block form above 438 drones: opted in once per device, for every size (as the tile kernels)
+    if (smem > 48 * 1024) {  // the block form above 438 drones
         static bool done[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        cudaError_t e = opt_in_shared((const void*)render_kernel<kCamThreads>, MDG_MAX_ENV_DRONES * kSceneF4 * sizeof(float4),
+                                      done);
         if (e != cudaSuccess) return e;
-        const bool known = dev >= 0 && dev < 64;
-        if (!known || !done[dev]) {
-            e = cudaFuncSetAttribute(render_kernel<kCamThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     MDG_MAX_ENV_DRONES * kSceneF4 * (int)sizeof(float4));
-            if (e != cudaSuccess) return e;
-            if (known) done[dev] = true;
-        }
     }
     const long long grid = (a.n + teams - 1) / teams;
     if (warp) render_kernel<32><<<(unsigned)grid, kCamThreads, smem, s>>>(a);

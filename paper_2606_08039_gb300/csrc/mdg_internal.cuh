@@ -40,6 +40,10 @@ __device__ __forceinline__ const T* after_wait(const T* p)
 }
 #endif
 cudaError_t launch_overlapped(const void* fn, int grid, int block, void** args, size_t smem, cudaStream_t s);
+// Opts a kernel in to its largest launch's shared memory, once per device (`done` is the kernel's own): the
+// limit belongs to the kernel and not to a launch, so that a launch that set it to its own size could lower
+// it under a larger one that another host thread is about to make.
+cudaError_t opt_in_shared(const void* kernel, size_t bytes, bool (&done)[64]);
 
 // Float32 copies of the model constants with the products the kernels need folded in
 // once on the host (in double precision, then rounded).

@@ -2360,9 +2360,20 @@ static void* step_kernel_ptr(int flags, int N, int block, bool pairs)
 static size_t features_smem_bytes(int B) { return obs_stage_offset(B) + (size_t)(B / 32) * kRawStage; }
 static size_t prepare_smem_bytes(int B) { return obs_stage_offset(B) + (size_t)(B / 32) * kInputStage; }
 
-// Opt the tile kernels in to the shared memory of the largest block, once per device: the limit
-// belongs to the kernel and not to a launch, so that a launch that set it to its own size could
-// lower it under a larger one that another host thread is about to make.
+cudaError_t opt_in_shared(const void* kernel, size_t bytes, bool (&done)[64])
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < 64;
+    if (known && done[dev]) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && known) done[dev] = true;
+    return e;
+}
+
+// Opt the step and observation kernels in to the shared memory of the largest block, once per device
+// (opt_in_shared, for all variants).
 static cudaError_t tile_kernels_setup()
 {
     static bool done[64] = {};
@@ -2379,11 +2390,7 @@ static cudaError_t tile_kernels_setup()
         return e;
     MDG_STEP_VARIANTS(MDG_ATTR)
 #undef MDG_ATTR
-    if ((e = cudaFuncSetAttribute(obs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)features_smem_bytes(1024))) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(surrogate_prepare_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)prepare_smem_bytes(1024))) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(obs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
         return e;
     if (dev >= 0 && dev < 64) done[dev] = true;
     return cudaSuccess;
@@ -2527,7 +2534,8 @@ cudaError_t launch_rollout(const RolloutArgs& r, int block, int uniform_flags, i
 cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s)
 {
     if (n_tiles == 0) return cudaSuccess;
-    cudaError_t e = tile_kernels_setup();
+    static bool done[64] = {};
+    cudaError_t e = opt_in_shared((const void*)features_kernel, features_smem_bytes(1024), done);
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<SurrogateArgs*>(&a)};
     return launch_overlapped((const void*)features_kernel, n_tiles, block, args, features_smem_bytes(block), s);
@@ -2536,7 +2544,8 @@ cudaError_t launch_features(const SurrogateArgs& a, int n_tiles, int block, cuda
 cudaError_t launch_surrogate_prepare(const SurrogateArgs& a, int n_tiles, int block, cudaStream_t s)
 {
     if (n_tiles == 0) return cudaSuccess;
-    cudaError_t e = tile_kernels_setup();
+    static bool done[64] = {};
+    cudaError_t e = opt_in_shared((const void*)surrogate_prepare_kernel, prepare_smem_bytes(1024), done);
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<SurrogateArgs*>(&a)};
     return launch_overlapped((const void*)surrogate_prepare_kernel, n_tiles, block, args, prepare_smem_bytes(block), s);
